@@ -171,6 +171,71 @@ __device__ __forceinline__ void rec_split(const float4* rec, float2 (&v)[2 * D])
   }
 }
 
+// One target against one source record (two sources) of StepForward.
+// q, p: the target, duplicated; v[k] = -q~_j, v[D + k] = p_j; aF += g p_j,
+// aG += c g d~.
+template <int D>
+__device__ __forceinline__ void fwd_record(const float2 (&q)[D], const float2 (&p)[D], const float2 (&v)[2 * D],
+                                           float2 (&aF)[D], float2 (&aG)[D]) {
+  float2 d[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) d[k] = __fadd2_rn(q[k], v[k]);
+  float2 r2 = __fmul2_rn(d[0], d[0]);
+#pragma unroll
+  for (int k = 1; k < D; ++k) r2 = __ffma2_rn(d[k], d[k], r2);
+  const float2 g = gauss2(r2);
+  float2 cc = __fmul2_rn(p[0], v[D]);
+#pragma unroll
+  for (int k = 1; k < D; ++k) cc = __ffma2_rn(p[k], v[D + k], cc);
+  const float2 w = __fmul2_rn(g, cc);
+#pragma unroll
+  for (int k = 0; k < D; ++k) aF[k] = __ffma2_rn(g, v[D + k], aF[k]);
+#pragma unroll
+  for (int k = 0; k < D; ++k) aG[k] = __ffma2_rn(w, d[k], aG[k]);
+}
+
+// One target against one source record of StepBackward.  v as above; w[k] =
+// alpha_j, w[D + k] = -b~_j.  With m_j = alpha_j + t p_j (which B needs
+// anyway), h = u + c t = alpha_i.p_j + p_i.m_j: 35 paired instructions instead
+// of the 36 that forming u and c t apart takes (the loop is bound by the FP32
+// pipe and its operand reads).  Whole gradients: 19.64 against 19.89 ms at
+// N = 16384 (T = 40), 998 against 1006 us at 4096 (T = 20).
+template <int D>
+__device__ __forceinline__ void bwd_record(const float2 (&q)[D], const float2 (&p)[D], const float2 (&a)[D],
+                                           const float2 (&b)[D], const float2 (&v)[2 * D], const float2 (&w)[2 * D],
+                                           float2 (&a1)[D], float2 (&a2)[D], float2 (&bb)[D]) {
+  float2 d[D], e[D], m[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) d[k] = __fadd2_rn(q[k], v[k]);
+  float2 r2 = __fmul2_rn(d[0], d[0]);
+#pragma unroll
+  for (int k = 1; k < D; ++k) r2 = __ffma2_rn(d[k], d[k], r2);
+  const float2 g = gauss2(r2);
+  float2 cc = __fmul2_rn(p[0], v[D]);
+#pragma unroll
+  for (int k = 1; k < D; ++k) cc = __ffma2_rn(p[k], v[D + k], cc);
+#pragma unroll
+  for (int k = 0; k < D; ++k) e[k] = __fadd2_rn(b[k], w[D + k]);
+  float2 t = __fmul2_rn(e[0], d[0]);
+#pragma unroll
+  for (int k = 1; k < D; ++k) t = __ffma2_rn(e[k], d[k], t);
+#pragma unroll
+  for (int k = 0; k < D; ++k) m[k] = __ffma2_rn(t, v[D + k], w[k]);
+  float2 h = __fmul2_rn(a[0], v[D]);
+#pragma unroll
+  for (int k = 1; k < D; ++k) h = __ffma2_rn(a[k], v[D + k], h);
+#pragma unroll
+  for (int k = 0; k < D; ++k) h = __ffma2_rn(p[k], m[k], h);
+  const float2 gc = __fmul2_rn(g, cc);
+  const float2 gh = __fmul2_rn(g, h);
+#pragma unroll
+  for (int k = 0; k < D; ++k) a1[k] = __ffma2_rn(gc, e[k], a1[k]);
+#pragma unroll
+  for (int k = 0; k < D; ++k) a2[k] = __ffma2_rn(gh, d[k], a2[k]);
+#pragma unroll
+  for (int k = 0; k < D; ++k) bb[k] = __ffma2_rn(g, m[k], bb[k]);
+}
+
 // ---------------------------------------------------------------- StepForward tile
 // Per target i:  Hp_i = sum_j g_ij p_j  and  G~_i = sum_j c_ij g_ij (q~_i - q~_j),
 // with Hq_i = -kappa G~_i.  D = 3 (or 2 for planar landmarks) coordinates.
@@ -211,21 +276,7 @@ struct FwdTile {
           rec_split<D>(Q + ((sb + jj) / 2 + u) * D, v);
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            float2 d[D];
-#pragma unroll
-            for (int k = 0; k < D; ++k) d[k] = __fadd2_rn(q[r][k], v[k]);
-            float2 r2 = __fmul2_rn(d[0], d[0]);
-#pragma unroll
-            for (int k = 1; k < D; ++k) r2 = __ffma2_rn(d[k], d[k], r2);
-            const float2 g = gauss2(r2);
-            float2 cc = __fmul2_rn(p[r][0], v[D]);
-#pragma unroll
-            for (int k = 1; k < D; ++k) cc = __ffma2_rn(p[r][k], v[D + k], cc);
-            const float2 w = __fmul2_rn(g, cc);
-#pragma unroll
-            for (int k = 0; k < D; ++k) aF[r][k] = __ffma2_rn(g, v[D + k], aF[r][k]);
-#pragma unroll
-            for (int k = 0; k < D; ++k) aG[r][k] = __ffma2_rn(w, d[k], aG[r][k]);
+            fwd_record<D>(q[r], p[r], v, aF[r], aG[r]);
           }
         }
       }
@@ -253,8 +304,8 @@ struct FwdTile {
 // Sources carry q~ = kq q, p (QP records) and alpha, b~ = kappa beta (AB
 // records).  Per pair:
 //   d~ = q~_i - q~_j, g = 2^-|d~|^2, c = p_i.p_j, e~ = b~_i - b~_j,
-//   t = e~.d~ (= s e.d), u = alpha_i.p_j + alpha_j.p_i, h = u + c t,
-//   A1 += g c e~,  A2 += g h d~,  B += g (alpha_j + t p_j);
+//   t = e~.d~ (= s e.d), m_j = alpha_j + t p_j, h = u + c t = alpha_i.p_j + p_i.m_j,
+//   A1 += g c e~,  A2 += g h d~,  B += g m_j;
 // dalpha = kq A1 - kappa A2 and dbeta = B.
 template <int R, int D = 3>
 struct BwdTile {
@@ -297,35 +348,7 @@ struct BwdTile {
           rec_split<D>(Ab + ri, w);
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            float2 d[D], e[D];
-#pragma unroll
-            for (int k = 0; k < D; ++k) d[k] = __fadd2_rn(q[r][k], v[k]);
-            float2 r2 = __fmul2_rn(d[0], d[0]);
-#pragma unroll
-            for (int k = 1; k < D; ++k) r2 = __ffma2_rn(d[k], d[k], r2);
-            const float2 g = gauss2(r2);
-            float2 cc = __fmul2_rn(p[r][0], v[D]);
-#pragma unroll
-            for (int k = 1; k < D; ++k) cc = __ffma2_rn(p[r][k], v[D + k], cc);
-#pragma unroll
-            for (int k = 0; k < D; ++k) e[k] = __fadd2_rn(b[r][k], w[D + k]);
-            float2 t = __fmul2_rn(e[0], d[0]);
-#pragma unroll
-            for (int k = 1; k < D; ++k) t = __ffma2_rn(e[k], d[k], t);
-            float2 uu = __fmul2_rn(a[r][0], v[D]);
-#pragma unroll
-            for (int k = 1; k < D; ++k) uu = __ffma2_rn(a[r][k], v[D + k], uu);
-#pragma unroll
-            for (int k = 0; k < D; ++k) uu = __ffma2_rn(w[k], p[r][k], uu);
-            const float2 h = __ffma2_rn(cc, t, uu);
-            const float2 gc = __fmul2_rn(g, cc);
-            const float2 gh = __fmul2_rn(g, h);
-#pragma unroll
-            for (int k = 0; k < D; ++k) a1[r][k] = __ffma2_rn(gc, e[k], a1[r][k]);
-#pragma unroll
-            for (int k = 0; k < D; ++k) a2[r][k] = __ffma2_rn(gh, d[k], a2[r][k]);
-#pragma unroll
-            for (int k = 0; k < D; ++k) bb[r][k] = __ffma2_rn(g, __ffma2_rn(t, v[D + k], w[k]), bb[r][k]);
+            bwd_record<D>(q[r], p[r], a[r], b[r], v, w, a1[r], a2[r], bb[r]);
           }
         }
       }
