@@ -425,57 +425,105 @@ gs_status get_graph(Workspace& w, const GraphKey& key, cudaGraphExec_t* out) {
   return GS_OK;
 }
 
-gs_status enqueue_gradient64(Workspace& w, const gs_params& prm, const float* dq, const double* p64_in,
-                             const float* dt, cudaStream_t st) {
+// Small problems go through one launch per call (small.cu).  The line: a forward
+// and a reverse step take 1.8 us at N = 64, 3.9 at 256, 7.5 at 512 in one launch
+// and 9.3 us by launches per step at 576 (8.4 at 256), whose gradient ends up
+// equally fast near 600 landmarks.  A caller who steers the step
+// kernels (a launch-shape override, the FP64 split combine, phase events)
+// gets the step kernels.
+static bool use_small(const Workspace& w, int npad, int J) {
+  return npad <= kSmallNpad && J <= kSmallSteps && !w.phase_timing && !step_override_set() && !combine_f64() &&
+         small_supported();
+}
+
+bool small_path(const Workspace& w, const gs_params& prm) {
+  return use_small(w, round_up(prm.N, kPad), stages_of(prm.integrator) * prm.T);
+}
+
+int shoot_ckpt(const Workspace& w, const gs_params& prm) {
+  return small_path(w, prm) ? 0 : effective_ckpt(prm.ckpt_every, prm.T);
+}
+
+gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const float* dq, const float* dp,
+                        const double* p64_in, const float* dt, const ShootOut& out, cudaStream_t st) {
   const int n = static_cast<int>(prm.N), dim = dim_of(prm);
   gs_status s = ensure_clean(w, n, st, dim);
   if (s != GS_OK) return s;
+  const KernelScales sc = make_scales(prm.sigma);
+  if (small_path(w, prm)) {
+    SmallArgs a;
+    a.q = dq;
+    a.p = dp;
+    a.p64_in = p64_in;
+    a.tgt = kind == 1 ? dt : nullptr;
+    a.kind = kind;
+    a.n = n;
+    a.npad = round_up(n, kPad);
+    a.T = prm.T;
+    a.groups = 0;
+    a.rk = prm.integrator == GS_RK4;
+    a.h_end = kind == 1 && prm.kinetic_at == GS_KINETIC_END;
+    a.dt = 1.0 / prm.T;
+    a.kq = sc.kq;
+    a.kappa = sc.kappa;
+    a.lambda = prm.lambda;
+    a.adj_scale = a.rk ? a.dt / 6.0 : 1.0;
+    a.traj = w.traj;
+    a.slot = w.slot();
+    a.q64 = w.q64;
+    a.p64 = w.p64;
+    a.t64 = kind == 1 ? w.t64 : nullptr;
+    a.out_a = out.a;
+    a.out_b = out.b;
+    a.gp64 = out.gp64;
+    a.scalars = w.scalars;
+    a.status = w.status;
+    GS_CUDA(launch_small_sweep(a, dim, st));
+    return GS_OK;
+  }
   PackArgs pk;
   pk.q = dq;
-  pk.p = nullptr;
+  pk.p = dp;
   pk.p64_in = p64_in;
   pk.tgt = dt;
   pk.q64 = w.q64;
   pk.p64 = w.p64;
-  pk.t64 = w.t64;
+  pk.t64 = kind == 1 ? w.t64 : nullptr;
   pk.qp = w.traj;
   pk.n = n;
-  pk.kq = make_scales(prm.sigma).kq;
+  pk.kq = sc.kq;
   pk.status = w.status;
   pk.dim = dim;
   GS_CUDA(launch_pack(pk, st));
   cudaGraphExec_t ge = nullptr;
-  const GraphKey key{1,           n, prm.T, prm.sigma, prm.lambda, effective_ckpt(prm.ckpt_every, prm.T), w.phase_timing,
-                     prm.integrator, prm.kinetic_at, dim};
+  const GraphKey key{kind,           n, prm.T, prm.sigma, kind == 1 ? prm.lambda : 0.0,
+                     kind == 1 ? effective_ckpt(prm.ckpt_every, prm.T) : 0, w.phase_timing,
+                     prm.integrator, kind == 1 ? prm.kinetic_at : 0, dim};
   if ((s = get_graph(w, key, &ge)) != GS_OK) return s;
   GS_CUDA(cudaGraphLaunch(ge, st));
+  // The graph leaves its results in the workspace.
+  const int n3 = dim * n;
+  if (kind == 0) {
+    if (out.a) GS_CUDA(launch_unpack(UnpackArgs{w.q64, out.a, n3}, st));
+    if (out.b) GS_CUDA(launch_unpack(UnpackArgs{w.p64, out.b, n3}, st));
+  } else {
+    const size_t bytes = n3 * sizeof(float);
+    if (out.a && out.a != w.out_a) GS_CUDA(cudaMemcpyAsync(out.a, w.out_a, bytes, cudaMemcpyDeviceToDevice, st));
+    if (out.b && out.b != w.out_b) GS_CUDA(cudaMemcpyAsync(out.b, w.out_b, bytes, cudaMemcpyDeviceToDevice, st));
+    if (out.gp64 && out.gp64 != w.gp64)
+      GS_CUDA(cudaMemcpyAsync(out.gp64, w.gp64, n3 * sizeof(double), cudaMemcpyDeviceToDevice, st));
+  }
   return GS_OK;
 }
 
-gs_status enqueue_forward64(Workspace& w, const gs_params& prm, const float* dq, const double* p64_in,
-                            cudaStream_t st) {
-  const int n = static_cast<int>(prm.N), dim = dim_of(prm);
-  gs_status s = ensure_clean(w, n, st, dim);
-  if (s != GS_OK) return s;
-  PackArgs pk;
-  pk.q = dq;
-  pk.p = nullptr;
-  pk.p64_in = p64_in;
-  pk.tgt = nullptr;
-  pk.q64 = w.q64;
-  pk.p64 = w.p64;
-  pk.t64 = nullptr;
-  pk.qp = w.traj;
-  pk.n = n;
-  pk.kq = make_scales(prm.sigma).kq;
-  pk.status = w.status;
-  pk.dim = dim;
-  GS_CUDA(launch_pack(pk, st));
-  cudaGraphExec_t ge = nullptr;
-  if ((s = get_graph(w, GraphKey{0, n, prm.T, prm.sigma, 0.0, 0, w.phase_timing, prm.integrator, 0, dim}, &ge)) !=
-      GS_OK)
-    return s;
-  GS_CUDA(cudaGraphLaunch(ge, st));
+// Where a call's kernels write a caller's output: the array itself when it is
+// this device's memory, else the staging buffer (copied out afterwards).
+static gs_status out_ptr(float* user, float* staging, float** dev) {
+  *dev = nullptr;
+  if (!user) return GS_OK;
+  const PtrKind kind = pointer_kind(user);
+  if (kind == kPtrOtherDevice) return other_device();
+  *dev = kind == kPtrDevice ? user : staging;
   return GS_OK;
 }
 
@@ -490,61 +538,31 @@ gs_status run_shoot(int kind, const gs_params* prm, const float* q0, const float
   if ((s = get_workspace(&w)) != GS_OK) return s;
   const int n = static_cast<int>(prm->N), T = prm->T;
   const int npad = round_up(n, kPad);
-  const int ckpt = kind == 1 ? effective_ckpt(prm->ckpt_every, T) : 0;
+  const int ckpt = kind == 1 ? shoot_ckpt(*w, *prm) : 0;
   if ((s = reserve(*w, npad, record_slots(T, ckpt, stages_of(prm->integrator)), 1, ckpt ? (T + ckpt - 1) / ckpt : 0)) !=
       GS_OK)
     return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int dim = dim_of(*prm);
-  if ((s = ensure_clean(*w, n, st, dim)) != GS_OK) return s;
   const size_t n3 = static_cast<size_t>(dim) * n;  // floats per (N, dim) array
   bool host = false;
   const float *dq = nullptr, *dp = nullptr, *dt = nullptr;
   if ((s = stage_in(q0, w->in_q, n3, st, &dq, &host)) != GS_OK) return s;
   if ((s = stage_in(p0, w->in_p, n3, st, &dp, &host)) != GS_OK) return s;
   if (kind == 1 && (s = stage_in(target, w->in_t, n3, st, &dt, &host)) != GS_OK) return s;
-  PackArgs pk;
-  pk.q = dq;
-  pk.p = dp;
-  pk.p64_in = nullptr;
-  pk.tgt = dt;
-  pk.q64 = w->q64;
-  pk.p64 = w->p64;
-  pk.t64 = kind == 1 ? w->t64 : nullptr;
-  pk.qp = w->traj;
-  pk.n = n;
-  pk.kq = make_scales(prm->sigma).kq;
-  pk.status = w->status;
-  pk.dim = dim;
-  GS_CUDA(launch_pack(pk, st));
-  cudaGraphExec_t ge = nullptr;
-  const GraphKey key{kind,           n, T, prm->sigma, kind == 1 ? prm->lambda : 0.0, ckpt, w->phase_timing,
-                     prm->integrator, kind == 1 ? prm->kinetic_at : 0, dim};
-  if ((s = get_graph(*w, key, &ge)) != GS_OK) return s;
-  GS_CUDA(cudaGraphLaunch(ge, st));
+  float* const ua = kind == 0 ? q1 : gp;
+  float* const ub = kind == 0 ? p1 : gq;
+  ShootOut out;
+  if ((s = out_ptr(ua, w->out_a, &out.a)) != GS_OK) return s;
+  if ((s = out_ptr(ub, w->out_b, &out.b)) != GS_OK) return s;
+  if ((s = enqueue_shoot(*w, kind, *prm, dq, dp, nullptr, dt, out, st)) != GS_OK) return s;
   bool want_sync = host;
-  if (kind == 0) {
-    if (q1) {
-      UnpackArgs u{w->q64, w->out_a, static_cast<int>(n3)};
-      GS_CUDA(launch_unpack(u, st));
-      if ((s = copy_out(q1, w->out_a, n3, st, &want_sync)) != GS_OK) return s;
-    }
-    if (p1) {
-      UnpackArgs u{w->p64, w->out_b, static_cast<int>(n3)};
-      GS_CUDA(launch_unpack(u, st));
-      if ((s = copy_out(p1, w->out_b, n3, st, &want_sync)) != GS_OK) return s;
-    }
-    if (H0) {
-      GS_CUDA(cudaMemcpyAsync(H0, w->scalars, sizeof(double), cudaMemcpyDeviceToHost, st));
-      want_sync = true;
-    }
-  } else {
-    if ((s = copy_out(gp, w->out_a, n3, st, &want_sync)) != GS_OK) return s;
-    if ((s = copy_out(gq, w->out_b, n3, st, &want_sync)) != GS_OK) return s;
-    if (loss) {
-      GS_CUDA(cudaMemcpyAsync(loss, w->scalars + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
-      want_sync = true;
-    }
+  if (ua && out.a != ua && (s = copy_out(ua, out.a, n3, st, &want_sync)) != GS_OK) return s;
+  if (ub && out.b != ub && (s = copy_out(ub, out.b, n3, st, &want_sync)) != GS_OK) return s;
+  double* const scalar = kind == 0 ? H0 : loss;
+  if (scalar) {
+    GS_CUDA(cudaMemcpyAsync(scalar, w->scalars + kind, sizeof(double), cudaMemcpyDeviceToHost, st));
+    want_sync = true;
   }
   if (want_sync) return finish_sync(*w, st);
   return GS_OK;
@@ -652,7 +670,10 @@ gs_status time_pair_kernels(const gs_params* prm, const float* q0, const float* 
   if (fwd_ms) *fwd_ms = m1 / reps;
   if (bwd_ms) *bwd_ms = m2 / reps;
   // pack, S launches per forward step, the terminal launch, S per reverse step
-  if (launches) *launches = 2 * stages_of(prm->integrator) * T + 1 + (prm->kinetic_at == GS_KINETIC_END ? 1 : 0);
+  // (small problems: one launch)
+  if (launches)
+    *launches = small_path(*w, *prm) ? 1
+                                     : 2 * stages_of(prm->integrator) * T + 1 + (prm->kinetic_at == GS_KINETIC_END ? 1 : 0);
   return finish_sync(*w, st);
 }
 

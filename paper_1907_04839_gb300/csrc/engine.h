@@ -142,13 +142,22 @@ gs_status copy_out(float* dst, const float* src, size_t n3, cudaStream_t st, boo
 gs_status finish_sync(Workspace& w, cudaStream_t st);
 gs_status check_params(const gs_params* prm);
 gs_status get_graph(Workspace& w, const GraphKey& key, cudaGraphExec_t* out);
-// Enqueue one gradient evaluation at FP64 momenta p64_in (device, N*3) with
-// q0 and target already on the device: pack, then replay the gradient graph.
-// Afterwards w.gp64 holds dL/dp0 and w.scalars[1] the loss (stream order).
-gs_status enqueue_gradient64(Workspace& w, const gs_params& prm, const float* dq, const double* p64_in,
-                             const float* dt, cudaStream_t st);
-// Enqueue the forward flow only at FP64 momenta; w.q64 then holds q(1).
-gs_status enqueue_forward64(Workspace& w, const gs_params& prm, const float* dq, const double* p64_in,
-                            cudaStream_t st);
+// Whether a flow or gradient of prm runs as one launch (small.cu), and the
+// checkpoint interval of its reverse sweep (0 on the small path, whose
+// trajectory is at most a few MB).
+bool small_path(const Workspace& w, const gs_params& prm);
+int shoot_ckpt(const Workspace& w, const gs_params& prm);
+// Device destinations of a sweep's results; null: not wanted.
+struct ShootOut {
+  float *a = nullptr, *b = nullptr;  // kind 0: q(1), p(1); kind 1: dL/dp0, dL/dq0
+  double* gp64 = nullptr;            // kind 1: FP64 dL/dp0
+};
+// Enqueue one forward flow (kind 0) or gradient (kind 1) from inputs on the
+// device: momenta from p64_in (FP64) when set, else from dp.  Afterwards, in
+// stream order, `out` is written, w.scalars[0] holds H0 (kind 0), w.scalars[1]
+// the loss (kind 1), w.q64 q(1) (kind 0), w.t64 the target (kind 1), and the record
+// slots the trajectory (Euler, no checkpoints).
+gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const float* dq, const float* dp,
+                        const double* p64_in, const float* dt, const ShootOut& out, cudaStream_t st);
 
 }  // namespace gs

@@ -219,6 +219,8 @@ constexpr int kVarBwdThreads = 64;
 // Override the fused step configuration of `kind` (threads == 0 restores the
 // built-in choice).  Returns false for an unknown variant.
 bool set_step_override(int kind, int threads, int R, int groups, int cluster);
+// Whether an override is installed for either kind.
+bool step_override_set();
 // Cluster scheduling preference forced on every step-kernel launch (0
 // driver default, 1 spread, 2 load balancing), or -1: each configuration's
 // own policy.
@@ -260,6 +262,36 @@ cudaError_t launch_bstep_forward(const StepConfig& cfg, int items, const StepFwd
                                  cudaStream_t st, bool pdl);
 cudaError_t launch_bstep_backward(const StepConfig& cfg, int items, const StepBwdArgs& a, const BatchTables& bt,
                                   cudaStream_t st, bool pdl);
+
+// ---------------------------------------------------------------- small problems
+// Up to kSmallNpad padded landmarks and kSmallSteps evaluations a sweep, one
+// launch of one 16-CTA cluster does a whole flow or gradient (small.cu).
+constexpr int kSmallNpad = 512;
+constexpr int kSmallSteps = 4096;
+
+struct SmallArgs {
+  const float* q;        // (N, dim) float32 inputs (device)
+  const float* p;        // may be null (zeros)
+  const double* p64_in;  // FP64 momenta (used instead of p when set)
+  const float* tgt;      // kind 1
+  int kind;              // 0 forward flow, 1 gradient
+  int n, npad, T;
+  int groups;            // source groups of a CTA (set by the launch)
+  int rk, h_end;
+  double dt, kq, kappa, lambda, adj_scale;
+  float4* traj;          // record slots 0 .. stages * T
+  size_t slot;           // float4 per slot
+  double *q64, *p64;     // kind 0: the end state
+  double* t64;           // kind 1: the FP64 targets
+  float *out_a, *out_b;  // kind 0: q(1), p(1); kind 1: dL/dp0, dL/dq0 (may be null)
+  double* gp64;          // FP64 copy of dL/dp0 (may be null)
+  double* scalars;       // as in StepFwdArgs
+  unsigned* status;
+};
+
+// Whether the current device can hold the cluster.
+bool small_supported();
+cudaError_t launch_small_sweep(const SmallArgs& a, int dim, cudaStream_t st);
 
 // ---------------------------------------------------------------- combine kernels
 struct PackArgs {

@@ -233,9 +233,10 @@ struct Lbfgs {
 
   // f and g at p0 = xv (device FP64); g goes to gv.  Synchronises.
   gs_status evaluate(const double* xv, double* gv, double* f) {
-    gs_status s = enqueue_gradient64(w, prm, dq, xv, dt, st);
+    ShootOut out;
+    out.gp64 = gv;
+    gs_status s = enqueue_shoot(w, 1, prm, dq, nullptr, xv, dt, out, st);
     if (s != GS_OK) return s;
-    GS_CUDA(cudaMemcpyAsync(gv, w.gp64, n3 * sizeof(double), cudaMemcpyDeviceToDevice, st));
     GS_CUDA(cudaMemcpyAsync(f, w.scalars + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
     ++evals;
     return finish_sync(w, st);
@@ -438,7 +439,7 @@ gs_status run_register(const gs_params* prm, const float* q0, const float* targe
   Workspace* w = nullptr;
   if ((s = get_workspace(&w)) != GS_OK) return s;
   const int n = static_cast<int>(prm->N), npad = round_up(n, kPad), n3 = dim_of(*prm) * n;
-  const int ckpt = effective_ckpt(prm->ckpt_every, prm->T);
+  const int ckpt = shoot_ckpt(*w, *prm);
   const int S = stages_of(prm->integrator);
   if ((s = reserve(*w, npad, std::max(S * prm->T, record_slots(prm->T, ckpt, S)), 1,
                    ckpt ? (prm->T + ckpt - 1) / ckpt : 0)) !=
@@ -460,7 +461,7 @@ gs_status run_register(const gs_params* prm, const float* q0, const float* targe
   bool dummy = false;
   if ((s = copy_out(p0_inout, w->out_a, n3, st, &dummy)) != GS_OK) return s;
   if (info) {
-    if ((s = enqueue_forward64(*w, *prm, dq, w->lb.x, st)) != GS_OK) return s;
+    if ((s = enqueue_shoot(*w, 0, *prm, dq, nullptr, w->lb.x, nullptr, ShootOut{}, st)) != GS_OK) return s;
     GS_CUDA(vlaunch(grid, st, k_dist, (const double*)w->q64, (const double*)w->t64, n, dim_of(*prm), w->lb.part,
                     w->lb.ticket,
                     w->lb.scal + kDots));

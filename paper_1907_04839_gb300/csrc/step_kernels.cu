@@ -787,6 +787,8 @@ bool set_step_override(int kind, int threads, int R, int groups, int cluster) {
   return true;
 }
 
+bool step_override_set() { return g_override[0][0] != 0 || g_override[1][0] != 0; }
+
 namespace {
 // One row of the measured step-configuration table: the padded landmark
 // count, then per kind (forward, reverse) the fastest CTA size and cluster

@@ -326,23 +326,7 @@ extern "C" gs_status flow_points(const gs_params* prm, const float* q0, const fl
   // The forward flow: record slot k of the trajectory holds the landmark
   // state of step k.
   const KernelScales sc = make_scales(prm->sigma);
-  PackArgs pk;
-  pk.q = dq;
-  pk.p = dp;
-  pk.p64_in = nullptr;
-  pk.tgt = nullptr;
-  pk.q64 = w->q64;
-  pk.p64 = w->p64;
-  pk.t64 = nullptr;
-  pk.qp = w->traj;
-  pk.n = n;
-  pk.kq = sc.kq;
-  pk.status = w->status;
-  pk.dim = 3;
-  GS_CUDA(launch_pack(pk, st));
-  cudaGraphExec_t ge = nullptr;
-  if ((s = get_graph(*w, GraphKey{0, n, T, prm->sigma, 0.0, 0, w->phase_timing}, &ge)) != GS_OK) return s;
-  GS_CUDA(cudaGraphLaunch(ge, st));
+  if ((s = enqueue_shoot(*w, 0, *prm, dq, dp, nullptr, nullptr, ShootOut{}, st)) != GS_OK) return s;
   // T Euler steps of the points, each with that step's landmark state.
   k_points_to64<<<conv_blocks(m3), 256, 0, st>>>(dx, w->pts64, m3);
   GS_CUDA(cudaGetLastError());
