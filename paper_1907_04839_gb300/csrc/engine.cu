@@ -60,6 +60,7 @@ gs_status get_workspace(Workspace** out) {
     w->device = dev;
     GS_CUDA(cudaDeviceGetAttribute(&w->num_sms, cudaDevAttrMultiProcessorCount, dev));
     GS_CUDA(cudaStreamCreateWithFlags(&w->capture_stream, cudaStreamNonBlocking));
+    GS_CUDA(cudaMallocHost(&w->host, 9 * sizeof(double)));
     it = g_ws.emplace(dev, w).first;
   }
   *out = it->second;
@@ -103,12 +104,11 @@ gs_status reserve(Workspace& w, int npad, int T, int splits, int nck) {
   GS_CUDA(dalloc(w, &w.out_b, n3));
   GS_CUDA(dalloc(w, &w.red_h, cr));
   GS_CUDA(dalloc(w, &w.red_m, cr));
-  GS_CUDA(dalloc(w, &w.scalars, 8));
+  GS_CUDA(dalloc(w, &w.scalars, 16));
+  w.status = reinterpret_cast<unsigned*>(w.scalars + 8);
   GS_CUDA(dalloc(w, &w.ticket, 8));
-  GS_CUDA(dalloc(w, &w.status, 8));
   GS_CUDA(cudaMemset(w.ticket, 0, 8 * sizeof(unsigned)));
-  GS_CUDA(cudaMemset(w.status, 0, 8 * sizeof(unsigned)));
-  GS_CUDA(cudaMemset(w.scalars, 0, 8 * sizeof(double)));
+  GS_CUDA(cudaMemset(w.scalars, 0, 16 * sizeof(double)));
   w.cap_npad = cn;
   w.cap_T = cT;
   w.cap_splits = cs;
@@ -186,9 +186,10 @@ gs_status copy_out(float* dst, const float* src, size_t n3, cudaStream_t st, boo
 
 // Read and clear the device status word (synchronises the stream).
 gs_status finish_sync(Workspace& w, cudaStream_t st) {
-  unsigned h = 0;
-  GS_CUDA(cudaMemcpyAsync(&h, w.status, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+  GS_CUDA(cudaMemcpyAsync(w.host, w.scalars, 9 * sizeof(double), cudaMemcpyDeviceToHost, st));
   GS_CUDA(cudaStreamSynchronize(st));
+  unsigned h = 0;
+  std::memcpy(&h, w.host + 8, sizeof(h));
   if (h) {
     cudaMemset(w.status, 0, sizeof(unsigned));
     if (h & kErrTimeout) return fail(GS_ETIMEOUT, "a device-side wait expired");
@@ -560,12 +561,10 @@ gs_status run_shoot(int kind, const gs_params* prm, const float* q0, const float
   if (ua && out.a != ua && (s = copy_out(ua, out.a, n3, st, &want_sync)) != GS_OK) return s;
   if (ub && out.b != ub && (s = copy_out(ub, out.b, n3, st, &want_sync)) != GS_OK) return s;
   double* const scalar = kind == 0 ? H0 : loss;
-  if (scalar) {
-    GS_CUDA(cudaMemcpyAsync(scalar, w->scalars + kind, sizeof(double), cudaMemcpyDeviceToHost, st));
-    want_sync = true;
-  }
-  if (want_sync) return finish_sync(*w, st);
-  return GS_OK;
+  if (!want_sync && !scalar) return GS_OK;
+  s = finish_sync(*w, st);
+  if (scalar) *scalar = w->host[kind];
+  return s;
 }
 
 gs_status run_step(int kind, int64_t N, double sigma, const float* q, const float* p, const float* alpha,
@@ -974,6 +973,7 @@ void gs_release_workspace(void) {
     for (cudaEvent_t& e : kv.second->phase)
       if (e) cudaEventDestroy(e);
     if (kv.second->capture_stream) cudaStreamDestroy(kv.second->capture_stream);
+    if (kv.second->host) cudaFreeHost(kv.second->host);
     delete kv.second;
     cudaSetDevice(cur);
   }

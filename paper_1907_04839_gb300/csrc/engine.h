@@ -92,7 +92,8 @@ struct Workspace {
   float *in_q = nullptr, *in_p = nullptr, *in_t = nullptr, *in_a = nullptr;
   float *out_a = nullptr, *out_b = nullptr;
   double *red_h = nullptr, *red_m = nullptr, *scalars = nullptr;
-  unsigned *ticket = nullptr, *status = nullptr;
+  unsigned *ticket = nullptr, *status = nullptr;  // status lies behind the 8 scalars:
+  double* host = nullptr;                         // one copy brings both here (pinned, 9 doubles)
   // The trajectory and adjoint records hold zero padding for this N and
   // dimension (key 4 N + dim; -1: unknown).
   int clean_n = -1;
@@ -139,6 +140,8 @@ gs_status ensure_clean(Workspace& w, int n, cudaStream_t st, int dim = 3);
 bool is_device_ptr(const void* p);
 gs_status stage_in(const float* src, float* staging, size_t n3, cudaStream_t st, const float** dev, bool* host);
 gs_status copy_out(float* dst, const float* src, size_t n3, cudaStream_t st, bool* host);
+// Wait for the stream; the scalars are in w.host afterwards, the status word
+// is read and cleared.
 gs_status finish_sync(Workspace& w, cudaStream_t st);
 gs_status check_params(const gs_params* prm);
 gs_status get_graph(Workspace& w, const GraphKey& key, cudaGraphExec_t* out);
