@@ -62,12 +62,15 @@ struct LbfgsBufs {
   std::vector<void*> allocs;
   double *x = nullptr, *g = nullptr, *d = nullptr, *xt = nullptr, *gt = nullptr;
   double *S = nullptr, *Y = nullptr;  // m x n3 each
-  double* scal = nullptr;             // alpha[m], beta, dots...
-  double* part = nullptr;             // per-CTA partial sums of a dot product
+  double* scal = nullptr;             // what the host reads back (lbfgs.cu)
+  double* host = nullptr;             // its pinned copy
+  double* part = nullptr;             // per-CTA partial sums of dot products
   unsigned* ticket = nullptr;
   void free_all() {
     for (void* p : allocs) cudaFree(p);
     allocs.clear();
+    if (host) cudaFreeHost(host);
+    host = nullptr;
     n3 = m = 0;
   }
 };

@@ -9,11 +9,17 @@
 //  * stop when ||g|| <= grad_tol ||g0||, or after max_iter iterations.
 //
 // The iterate, the gradient, the direction and the (s, y) history are FP64
-// vectors on the device.  Dot products reduce deterministically: per-CTA
-// partials, then the last CTA adds them in a fixed order.  The host runs the
-// scalar control flow of the line search.  Each evaluation is one replay of
-// the gradient graph at FP64 momenta, which returns the loss and
-// phi'(a) = g.d to the host.
+// vectors on the device.  Dot products reduce deterministically, in a fixed
+// order.  The host runs the scalar control flow of the line search.  An
+// iteration is three launches around its evaluation and one readback: the
+// direction with the step to the first trial point (one cluster), the sweeps,
+// and every product the host may need of the result.  The first trial of
+// an iteration is evaluated before the host has seen its slope; the rare
+// direction that does not descend is thrown away with its evaluation.
+//
+// A registration at N = 256, T = 10, 8 iterations: 950 us; 2.70 ms with a launch
+// and a copy per operation of the recursion, a synchronising copy per scalar
+// and the gradient by launches per step.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -26,82 +32,195 @@ namespace gs {
 namespace {
 
 constexpr int kLT = 256;     // threads per CTA of the vector kernels
-constexpr int kMaxDots = 4;  // dot products computed in one pass
 constexpr int kMaxM = 64;
-
-// scal[] slots
-constexpr int kAlpha = 0;             // alpha[m]
-constexpr int kDots = kMaxM + 1;      // results of the last k_dots pass (kMaxM: spare)
 
 int vec_grid(int n, int num_sms) { return std::max(1, std::min((n + kLT - 1) / kLT, 2 * num_sms)); }
 
-struct DotArgs {
-  const double* a[kMaxDots];
-  const double* b[kMaxDots];
-  int count;
+// What the host reads back after an evaluation.
+enum : int { kRbSlope, kRbSy, kRbYy, kRbSs, kRbGg, kRbLoss, kRbSlope0, kRbStatus, kRbWords };
+
+struct EvalArgs {
+  const double *x, *g, *d, *xt, *gt;
   int n;
-  double mult[kMaxDots];
-  double* part;       // [count][gridDim.x]
+  double* part;            // [kRbLoss][gridDim.x]
   unsigned* ticket;
-  double* out;        // out[k] = mult[k] * a[k].b[k]
+  const double* loss;
+  const unsigned* status;
+  double* out;             // kRbWords (kRbSlope0 is k_direction's)
 };
 
-// Up to four dot products in one pass, reduced deterministically.
-__global__ void __launch_bounds__(kLT) k_dots(DotArgs d) {
-  __shared__ double sh[kLT / 32];
+// The products of an evaluated trial point (xt, gt): its slope gt.d, and with
+// s = xt - x, y = gt - g the numbers s.y, y.y, s.s and gt.gt that follow an
+// accepted step.  One pass; the last CTA adds the partials in order.
+__global__ void __launch_bounds__(kLT) k_eval_products(EvalArgs e) {
+  constexpr int K = kRbLoss;
+  __shared__ double sh[K][kLT / 32];
   __shared__ int am_last;
-  double v[kMaxDots] = {0.0, 0.0, 0.0, 0.0};
-  for (int i = blockIdx.x * kLT + threadIdx.x; i < d.n; i += gridDim.x * kLT) {
-#pragma unroll
-    for (int k = 0; k < kMaxDots; ++k)
-      if (k < d.count) v[k] = fma(d.a[k][i], d.b[k][i], v[k]);
+  double v[K] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int i = blockIdx.x * kLT + threadIdx.x; i < e.n; i += gridDim.x * kLT) {
+    const double gt = e.gt[i], s = e.xt[i] - e.x[i], y = gt - e.g[i];
+    v[kRbSlope] = fma(gt, e.d[i], v[kRbSlope]);
+    v[kRbSy] = fma(s, y, v[kRbSy]);
+    v[kRbYy] = fma(y, y, v[kRbYy]);
+    v[kRbSs] = fma(s, s, v[kRbSs]);
+    v[kRbGg] = fma(gt, gt, v[kRbGg]);
   }
 #pragma unroll
-  for (int k = 0; k < kMaxDots; ++k) {
-    if (k >= d.count) break;
-    const double bs = block_sum_f64(v[k], sh);
-    if (threadIdx.x == 0) d.part[k * gridDim.x + blockIdx.x] = bs;
-  }
-  if (threadIdx.x == 0) {
+  for (int k = 0; k < K; ++k) v[k] = warp_sum_f64(v[k]);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (l == 0)
+#pragma unroll
+    for (int k = 0; k < K; ++k) sh[k][w] = v[k];
+  __syncthreads();
+  if (w == 0) {
+    if (l < K) {
+      double t = 0.0;
+      for (int u = 0; u < kLT / 32; ++u) t += sh[l][u];
+      e.part[l * gridDim.x + blockIdx.x] = t;
+    }
     __threadfence();
-    am_last = (atomicAdd(d.ticket, 1u) == gridDim.x - 1);
+    __syncwarp();
+    if (l == 0) am_last = (atomicAdd(e.ticket, 1u) == gridDim.x - 1);
   }
   __syncthreads();
-  if (!am_last || threadIdx.x >= 32) return;
+  if (!am_last || w >= K) return;
   __threadfence();
-  for (int k = 0; k < d.count; ++k) {
-    double t = 0.0;
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) t += *((volatile double*)&d.part[k * gridDim.x + b]);
-    t = warp_sum_f64(t);
-    if (threadIdx.x == 0) d.out[k] = d.mult[k] * t;
+  double t = 0.0;
+  for (unsigned b = l; b < gridDim.x; b += 32) t += *((volatile double*)&e.part[w * gridDim.x + b]);
+  t = warp_sum_f64(t);
+  if (l == 0) e.out[w] = t;
+  if (threadIdx.x == 0) {
+    e.out[kRbLoss] = *e.loss;
+    e.out[kRbStatus] = static_cast<double>(*e.status);
+    *e.ticket = 0u;
   }
-  if (threadIdx.x == 0) *d.ticket = 0u;
 }
 
-// y <- y + (c0 + c1 * sa[0] + c2 * sb[0]) x   (sa, sb device scalars or null)
-__global__ void __launch_bounds__(kLT) k_axpy(double* y, const double* x, int n, double c0, double c1,
-                                             const double* sa, double c2, const double* sb) {
-  const double coef = c0 + (sa ? c1 * sa[0] : 0.0) + (sb ? c2 * sb[0] : 0.0);
-  for (int i = blockIdx.x * kLT + threadIdx.x; i < n; i += gridDim.x * kLT) y[i] = fma(coef, x[i], y[i]);
-}
+constexpr int kDT = 512;  // threads per CTA of k_direction
+constexpr int kDC = 16;   // CTAs of its cluster
 
-// y <- c x
-__global__ void __launch_bounds__(kLT) k_scale(double* y, const double* x, int n, double c) {
-  for (int i = blockIdx.x * kLT + threadIdx.x; i < n; i += gridDim.x * kLT) y[i] = c * x[i];
+enum : int { kAcceptNone = 0, kAcceptStep = 1, kAcceptGrad = 2 };
+
+struct DirArgs {
+  double *x, *g, *d, *xt;
+  const double* gt;
+  double *S, *Y;           // m x n history
+  int n, m;
+  int accept;              // kAcceptStep: x <- xt, g <- gt; kAcceptGrad: g <- gt
+  int slot;                // with kAcceptStep: history slot of (xt - x, gt - g), -1: not kept
+  int direction;           // 0: accept only
+  int head, stored;        // the newest `stored` pairs end before slot `head`
+  double gamma;
+  double a1;               // xt <- x + a1 d
+  double* slope;           // g.d
+  double rho[kMaxM];
+};
+
+// Accept the last trial point, then d = -H g by the two-loop recursion, its
+// slope and the first trial point.  One cluster: a recursion of `stored` pairs
+// is 2 stored + 1 passes over d, each ended by a cluster-wide dot product, and
+// every pass updates d with one pair and multiplies it with the next, so a
+// pair costs two passes instead of four launches and a copy (N = 256, 7
+// pairs: 28 launches and 8 copies before).  Each element is read and written
+// by one thread throughout; only the dot products cross threads.
+__global__ void __launch_bounds__(kDT) k_direction(DirArgs a) {
+  __shared__ double sh[kDT / 32];
+  __shared__ double peers[2][kDC];  // every CTA's partial, two passes in turn
+  __shared__ double total;
+  __shared__ double alpha[kMaxM];
+  const int rank = static_cast<int>(cluster_rank());
+  if (blockDim.x != kDT || cluster_size() != kDC) return;
+  const int t0 = rank * kDT + threadIdx.x, step = kDC * kDT;
+  int turn = 0;
+  const auto cluster_total = [&](double v) -> double {
+    v = block_sum_f64(v, sh);
+    if (threadIdx.x < kDC) {
+      // thread c of warp 0 sends to CTA c (block_sum leaves the sum in warp 0)
+      v = __shfl_sync(0xffffu, v, 0);
+      const uint32_t to = dsmem_addr(smem_u32(&peers[turn][rank]), threadIdx.x);
+      asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(to), "d"(v) : "memory");
+    }
+    __syncwarp();
+    cluster_sync();
+    if (threadIdx.x < 32) {
+      double p = threadIdx.x < kDC ? peers[turn][threadIdx.x] : 0.0;
+      p = warp_sum_f64(p);
+      if (threadIdx.x == 0) total = p;
+    }
+    __syncthreads();
+    turn ^= 1;  // the next pass's stores may arrive while a slow CTA still reads this one's
+    return total;
+  };
+  const auto pair = [&](int k) { return (a.head - 1 - k + a.m) % a.m; };
+  cluster_sync();  // every CTA has started
+  for (int i = t0; i < a.n; i += step) {
+    double g = a.g[i];
+    if (a.accept) {
+      const double gt = a.gt[i];
+      if (a.accept == kAcceptStep) {
+        const double xt = a.xt[i];
+        if (a.slot >= 0) {
+          a.S[static_cast<size_t>(a.slot) * a.n + i] = xt - a.x[i];
+          a.Y[static_cast<size_t>(a.slot) * a.n + i] = gt - g;
+        }
+        a.x[i] = xt;
+      }
+      a.g[i] = g = gt;
+    }
+    if (a.direction) a.d[i] = g;
+  }
+  if (!a.direction) return;  // no peer reads this CTA's shared memory
+  const auto hist = [&](const double* h, int j) { return h + static_cast<size_t>(j) * a.n; };
+  // d <- d - alpha_j Y_j, newest pair first
+  double v = 0.0;
+  if (a.stored > 0) {
+    const double* S = hist(a.S, pair(0));
+    for (int i = t0; i < a.n; i += step) v = fma(S[i], a.d[i], v);
+  }
+  for (int k = 0; k < a.stored; ++k) {
+    const int j = pair(k);
+    const double al = a.rho[j] * cluster_total(v);
+    if (threadIdx.x == 0) alpha[j] = al;
+    const double* Y = hist(a.Y, j);
+    // next: the older pair's S, or (d scaled by gamma) the oldest pair's Y
+    const bool lastp = k + 1 == a.stored;
+    const double* N = lastp ? Y : hist(a.S, pair(k + 1));
+    const double sc = lastp ? a.gamma : 1.0;
+    v = 0.0;
+    for (int i = t0; i < a.n; i += step) {
+      const double d = sc * fma(-al, Y[i], a.d[i]);
+      a.d[i] = d;
+      v = fma(N[i], d, v);
+    }
+  }
+  __syncthreads();
+  for (int k = a.stored - 1; k >= 0; --k) {
+    const int j = pair(k);
+    const double c = alpha[j] - a.rho[j] * cluster_total(v);
+    const double* S = hist(a.S, j);
+    const double* N = k > 0 ? hist(a.Y, pair(k - 1)) : nullptr;
+    v = 0.0;
+    for (int i = t0; i < a.n; i += step) {
+      const double d = fma(c, S[i], a.d[i]);
+      a.d[i] = d;
+      if (N) v = fma(N[i], d, v);
+    }
+  }
+  v = 0.0;
+  for (int i = t0; i < a.n; i += step) {
+    const double d = -a.d[i];
+    a.d[i] = d;
+    a.xt[i] = fma(a.a1, d, a.x[i]);
+    v = fma(a.g[i], d, v);
+  }
+  v = cluster_total(v);
+  if (rank == 0 && threadIdx.x == 0) *a.slope = v;
+  // The last remote store of the kernel came before the last cluster barrier.
 }
 
 // xt <- x + a d
 __global__ void __launch_bounds__(kLT) k_step(double* xt, const double* x, const double* d, int n, double a) {
   for (int i = blockIdx.x * kLT + threadIdx.x; i < n; i += gridDim.x * kLT) xt[i] = fma(a, d[i], x[i]);
-}
-
-// s <- xt - x, y <- gt - g
-__global__ void __launch_bounds__(kLT) k_pair(double* s, double* y, const double* xt, const double* x,
-                                             const double* gt, const double* g, int n) {
-  for (int i = blockIdx.x * kLT + threadIdx.x; i < n; i += gridDim.x * kLT) {
-    s[i] = xt[i] - x[i];
-    y[i] = gt[i] - g[i];
-  }
 }
 
 __global__ void __launch_bounds__(kLT) k_f32_to_f64(double* y, const float* x, int n) {
@@ -183,14 +302,18 @@ gs_status alloc_lbfgs(Workspace& w, int n3, int m) {
   GS_CUDA(get(&b.gt, n));
   GS_CUDA(get(&b.S, n * m));
   GS_CUDA(get(&b.Y, n * m));
-  GS_CUDA(get(&b.scal, kMaxM + 16));
-  GS_CUDA(get(&b.part, kMaxDots * 4 * 1024));
+  GS_CUDA(get(&b.scal, 16));
+  GS_CUDA(get(&b.part, 4 * 4 * 1024));
   double* t = nullptr;
   GS_CUDA(get(&t, 8));
   b.ticket = reinterpret_cast<unsigned*>(t);
   GS_CUDA(cudaMemset(b.ticket, 0, 8 * sizeof(double)));
   GS_CUDA(cudaMemset(b.S, 0, n * m * sizeof(double)));
   GS_CUDA(cudaMemset(b.Y, 0, n * m * sizeof(double)));
+  // every vector starts finite: a product of an unused one is read back unused
+  for (double* p : {b.x, b.g, b.d, b.xt, b.gt}) GS_CUDA(cudaMemset(p, 0, n * sizeof(double)));
+  GS_CUDA(cudaDeviceSynchronize());  // the caller's stream need not wait for the default one
+  if (!b.host) GS_CUDA(cudaMallocHost(&b.host, 16 * sizeof(double)));
   b.n3 = n3;
   b.m = m;
   return GS_OK;
@@ -210,47 +333,45 @@ struct Lbfgs {
       : w(w_), prm(p), st(s), dq(q), dt(t), n3(static_cast<int>(dim_of(p) * p.N)), m(p.lbfgs_m),
         grid(vec_grid(n3, w_.num_sms)) {}
 
-  gs_status dots(int count, const double* const* a, const double* const* b, const double* mult, double* host) {
-    DotArgs d;
-    std::memset(&d, 0, sizeof(d));
-    for (int k = 0; k < count; ++k) {
-      d.a[k] = a[k];
-      d.b[k] = b[k];
-      d.mult[k] = mult ? mult[k] : 1.0;
-    }
-    d.count = count;
-    d.n = n3;
-    d.part = w.lb.part;
-    d.ticket = w.lb.ticket;
-    d.out = w.lb.scal + kDots;
-    GS_CUDA(vlaunch(grid, st, k_dots, d));
-    if (host) {
-      GS_CUDA(cudaMemcpyAsync(host, w.lb.scal + kDots, count * sizeof(double), cudaMemcpyDeviceToHost, st));
-      GS_CUDA(cudaStreamSynchronize(st));
-    }
+  // Enqueue the evaluation of the momenta xv: gradient to gt, products to scal.
+  gs_status enqueue_eval(const double* xv) {
+    LbfgsBufs& b = w.lb;
+    ShootOut out;
+    out.gp64 = b.gt;
+    gs_status s = enqueue_shoot(w, 1, prm, dq, nullptr, xv, dt, out, st);
+    if (s != GS_OK) return s;
+    const EvalArgs e{b.x, b.g, b.d, b.xt, b.gt, n3, b.part, b.ticket, w.scalars + 1, w.status, b.scal};
+    GS_CUDA(vlaunch(grid, st, k_eval_products, e));
     return GS_OK;
   }
 
-  // f and g at p0 = xv (device FP64); g goes to gv.  Synchronises.
-  gs_status evaluate(const double* xv, double* gv, double* f) {
-    ShootOut out;
-    out.gp64 = gv;
-    gs_status s = enqueue_shoot(w, 1, prm, dq, nullptr, xv, dt, out, st);
-    if (s != GS_OK) return s;
-    GS_CUDA(cudaMemcpyAsync(f, w.scalars + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
+  // Wait for the evaluation; its products are in w.lb.host afterwards.
+  gs_status readback() {
+    GS_CUDA(cudaMemcpyAsync(w.lb.host, w.lb.scal, kRbWords * sizeof(double), cudaMemcpyDeviceToHost, st));
+    GS_CUDA(cudaStreamSynchronize(st));
+    return GS_OK;
+  }
+
+  // Count the evaluation read back last; its errors.
+  gs_status count_eval() {
     ++evals;
-    return finish_sync(w, st);
+    return w.lb.host[kRbStatus] != 0.0 ? finish_sync(w, st) : GS_OK;
   }
 
   // phi(a) = f(x + a d) and phi'(a) = g(x + a d).d; the point and its
-  // gradient land in xt, gt.
-  gs_status eval_step(double a, double* f, double* dphi) {
-    GS_CUDA(vlaunch(grid, st, k_step, w.lb.xt, w.lb.x, w.lb.d, n3, a));
-    gs_status s = evaluate(w.lb.xt, w.lb.gt, f);
-    if (s != GS_OK) return s;
-    const double* A[1] = {w.lb.gt};
-    const double* B[1] = {w.lb.d};
-    return dots(1, A, B, nullptr, dphi);
+  // gradient land in xt, gt.  first: the evaluation that followed the
+  // direction, already read back.
+  gs_status eval_step(double a, bool first, double* f, double* dphi) {
+    gs_status s;
+    if (!first) {
+      GS_CUDA(vlaunch(grid, st, k_step, w.lb.xt, w.lb.x, w.lb.d, n3, a));
+      if ((s = enqueue_eval(w.lb.xt)) != GS_OK) return s;
+      if ((s = readback()) != GS_OK) return s;
+    }
+    if ((s = count_eval()) != GS_OK) return s;
+    *f = w.lb.host[kRbLoss];
+    *dphi = w.lb.host[kRbSlope];
+    return GS_OK;
   }
 
   static double cubic_min(double a, double fa, double da, double b, double fb, double db) {
@@ -273,7 +394,7 @@ struct Lbfgs {
     double a_prev = 0.0, f_prev = f0, d_prev = dphi0, a = a1;
     for (int it = 0; used < max_evals; ++it) {
       double fa, da;
-      gs_status s = eval_step(a, &fa, &da);
+      gs_status s = eval_step(a, used == 0, &fa, &da);
       if (s != GS_OK) return s;
       ++used;
       bool zoom = false;
@@ -297,7 +418,7 @@ struct Lbfgs {
           const double b1 = wdt > 0 ? hi - 0.1 * wdt : lo + 0.1 * wdt;
           if (!(aj >= std::min(b0, b1) && aj <= std::max(b0, b1))) aj = 0.5 * (lo + hi);
           double fj, dj;
-          s = eval_step(aj, &fj, &dj);
+          s = eval_step(aj, false, &fj, &dj);
           if (s != GS_OK) return s;
           ++used;
           if (!(fj <= f0 + c1 * aj * dphi0) || fj >= flo) {
@@ -322,98 +443,96 @@ struct Lbfgs {
     return GS_OK;
   }
 
-  // d = -H g by the two-loop recursion over the `stored` newest pairs.
-  gs_status direction(int head, int stored, const double* rho, double gamma) {
-    LbfgsBufs& b = w.lb;
-    GS_CUDA(cudaMemcpyAsync(b.d, b.g, n3 * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    for (int k = 0; k < stored; ++k) {
-      const int j = (head - 1 - k + m) % m;
-      const double* A[1] = {b.S + static_cast<size_t>(j) * n3};
-      const double* B[1] = {b.d};
-      const double mult[1] = {rho[j]};
-      gs_status s = dots(1, A, B, mult, nullptr);
-      if (s != GS_OK) return s;
-      GS_CUDA(cudaMemcpyAsync(b.scal + kAlpha + j, b.scal + kDots, sizeof(double), cudaMemcpyDeviceToDevice, st));
-      GS_CUDA(vlaunch(grid, st, k_axpy, b.d, b.Y + static_cast<size_t>(j) * n3, n3, 0.0, -1.0,
-                      (const double*)(b.scal + kAlpha + j), 0.0, (const double*)nullptr));
-    }
-    if (stored > 0) GS_CUDA(vlaunch(grid, st, k_scale, b.d, (const double*)b.d, n3, gamma));
-    for (int k = stored - 1; k >= 0; --k) {
-      const int j = (head - 1 - k + m) % m;
-      const double* A[1] = {b.Y + static_cast<size_t>(j) * n3};
-      const double* B[1] = {b.d};
-      const double mult[1] = {rho[j]};
-      gs_status s = dots(1, A, B, mult, nullptr);
-      if (s != GS_OK) return s;
-      GS_CUDA(vlaunch(grid, st, k_axpy, b.d, (const double*)(b.S + static_cast<size_t>(j) * n3), n3, 0.0, 1.0,
-                      (const double*)(b.scal + kAlpha + j), -1.0, (const double*)(b.scal + kDots)));
-    }
-    GS_CUDA(vlaunch(grid, st, k_scale, b.d, (const double*)b.d, n3, -1.0));
+  gs_status launch_direction(const DirArgs& a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kDC);
+    cfg.blockDim = dim3(kDT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kDC;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    GS_CUDA(cudaFuncSetAttribute(k_direction, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    GS_CUDA(cudaLaunchKernelEx(&cfg, k_direction, a));
     return GS_OK;
   }
 
   gs_status run(gs_register_info* info) {
     LbfgsBufs& b = w.lb;
-    double rho[kMaxM] = {0.0};
     int head = 0, stored = 0, status = 1, it = 0;
-    double gamma = 1.0, f = 0.0;
-    gs_status s = evaluate(b.x, b.g, &f);
+    DirArgs da;
+    std::memset(&da, 0, sizeof(da));
+    da.x = b.x;
+    da.g = b.g;
+    da.d = b.d;
+    da.xt = b.xt;
+    da.gt = b.gt;
+    da.S = b.S;
+    da.Y = b.Y;
+    da.n = n3;
+    da.m = m;
+    da.gamma = 1.0;
+    da.slope = b.scal + kRbSlope0;
+    da.accept = kAcceptGrad;
+    da.slot = -1;
+    gs_status s = enqueue_eval(b.x);
     if (s != GS_OK) return s;
-    double gg = 0.0;
-    {
-      const double* A[1] = {b.g};
-      const double* B[1] = {b.g};
-      if ((s = dots(1, A, B, nullptr, &gg)) != GS_OK) return s;
-    }
-    const double g0 = std::sqrt(gg);
+    if ((s = readback()) != GS_OK) return s;
+    if ((s = count_eval()) != GS_OK) return s;
+    double f = b.host[kRbLoss];
+    const double g0 = std::sqrt(b.host[kRbGg]);
     double gnorm = g0;
     if (g0 == 0.0) status = 0;
     for (it = 0; status == 1 && it < prm.max_iter; ++it) {
-      if ((s = direction(head, stored, rho, gamma)) != GS_OK) return s;
-      double dphi0 = 0.0;
-      {
-        const double* A[1] = {b.g};
-        const double* B[1] = {b.d};
-        if ((s = dots(1, A, B, nullptr, &dphi0)) != GS_OK) return s;
-      }
+      da.direction = 1;
+      da.head = head;
+      da.stored = stored;
+      da.a1 = (it == 0) ? 1.0 / g0 : 1.0;
+      if ((s = launch_direction(da)) != GS_OK) return s;
+      if ((s = enqueue_eval(b.xt)) != GS_OK) return s;
+      if ((s = readback()) != GS_OK) return s;
+      da.accept = kAcceptNone;
+      double dphi0 = b.host[kRbSlope0];
       if (!(dphi0 < 0.0)) {  // not a descent direction: restart from -g
-        GS_CUDA(vlaunch(grid, st, k_scale, b.d, (const double*)b.g, n3, -1.0));
+        if (static_cast<unsigned>(b.host[kRbStatus]) & kErrNonFinite)
+          GS_CUDA(cudaMemsetAsync(w.status, 0, sizeof(unsigned), st));  // of the point thrown away
         dphi0 = -gnorm * gnorm;
-        stored = 0;
+        da.stored = stored = 0;
+        if ((s = launch_direction(da)) != GS_OK) return s;
+        if ((s = enqueue_eval(b.xt)) != GS_OK) return s;
+        if ((s = readback()) != GS_OK) return s;
       }
-      const double a1 = (it == 0) ? 1.0 / g0 : 1.0;
       double a = 0.0, fn = 0.0;
-      if ((s = line_search(f, dphi0, a1, &a, &fn)) != GS_OK) return s;
+      if ((s = line_search(f, dphi0, da.a1, &a, &fn)) != GS_OK) return s;
       if (a == 0.0) {
         status = 2;  // no step met the Wolfe conditions: noise floor reached
         break;
       }
-      double* sv = b.S + static_cast<size_t>(head) * n3;
-      double* yv = b.Y + static_cast<size_t>(head) * n3;
-      GS_CUDA(vlaunch(grid, st, k_pair, sv, yv, (const double*)b.xt, (const double*)b.x, (const double*)b.gt,
-                      (const double*)b.g, n3));
-      double r4[4];
-      {
-        const double* A[4] = {sv, yv, sv, b.gt};
-        const double* B[4] = {yv, yv, sv, b.gt};
-        if ((s = dots(4, A, B, nullptr, r4)) != GS_OK) return s;
-      }
-      const double sy = r4[0], yy = r4[1], ss = r4[2];
+      // The accepted point is the one evaluated last.
+      const double sy = b.host[kRbSy], yy = b.host[kRbYy], ss = b.host[kRbSs];
+      da.accept = kAcceptStep;
+      da.slot = -1;
       if (sy > 1e-12 * std::sqrt(ss * yy)) {
-        rho[head] = 1.0 / sy;
-        gamma = sy / yy;
+        da.slot = head;
+        da.rho[head] = 1.0 / sy;
+        da.gamma = sy / yy;
         head = (head + 1) % m;
         if (stored < m) ++stored;
       }
-      GS_CUDA(cudaMemcpyAsync(b.x, b.xt, n3 * sizeof(double), cudaMemcpyDeviceToDevice, st));
-      GS_CUDA(cudaMemcpyAsync(b.g, b.gt, n3 * sizeof(double), cudaMemcpyDeviceToDevice, st));
       f = fn;
-      gnorm = std::sqrt(r4[3]);
+      gnorm = std::sqrt(b.host[kRbGg]);
       if (gnorm <= prm.grad_tol * g0) {
         status = 0;
         ++it;
         break;
       }
+    }
+    if (da.accept == kAcceptStep) {  // the last step's x
+      da.direction = 0;
+      if ((s = launch_direction(da)) != GS_OK) return s;
     }
     if (info) {
       info->loss = f;
@@ -463,10 +582,9 @@ gs_status run_register(const gs_params* prm, const float* q0, const float* targe
   if (info) {
     if ((s = enqueue_shoot(*w, 0, *prm, dq, nullptr, w->lb.x, nullptr, ShootOut{}, st)) != GS_OK) return s;
     GS_CUDA(vlaunch(grid, st, k_dist, (const double*)w->q64, (const double*)w->t64, n, dim_of(*prm), w->lb.part,
-                    w->lb.ticket,
-                    w->lb.scal + kDots));
-    double dist[2] = {0.0, 0.0};
-    GS_CUDA(cudaMemcpyAsync(dist, w->lb.scal + kDots, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+                    w->lb.ticket, w->lb.scal));
+    double* const dist = w->lb.host;
+    GS_CUDA(cudaMemcpyAsync(dist, w->lb.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
     if ((s = finish_sync(*w, st)) != GS_OK) return s;
     info->avg_dist = dist[0] / n;
     info->max_dist = dist[1];
