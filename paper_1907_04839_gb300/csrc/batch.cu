@@ -37,11 +37,54 @@
 namespace gs {
 namespace {
 
-constexpr int kBT = 256;     // threads of the per-problem kernels
+// Threads of the per-problem kernels.  One CTA does a problem's O(N) work, so
+// it is bound by the latency of its passes: 1024 threads instead of 256 keep
+// four times the loads in flight.
+constexpr int kBT = 1024;
 constexpr int kMaxM = 64;
 
 // ---------------------------------------------------------------- per-problem kernels
 // One CTA per listed problem (blockIdx.x indexes `list`).
+
+// A problem's segment at admission: its inputs (FP32, staged where gt and xt
+// will be, which every evaluation writes before anything reads them) to t64
+// and x in FP64, everything else of it to zero (record padding must
+// be exactly zero, and no earlier problem's value may show).  blockIdx.y is
+// the row: a record slot, an FP64 vector, a history vector or the input
+// padding.  One launch instead of a memset per row (T + 2m + 15 of them).
+constexpr int kNumVecs = 11;
+struct AdmitArgs {
+  float4 *traj, *adj;
+  size_t slot, r0, rl;  // record slots: float4 per slot, the segment's range
+  int slots;
+  double* vec[kNumVecs];  // [0] = x, [1] = t64
+  double *S, *Y;
+  size_t stride, b3;
+  int m, n3, e3;          // inputs and padded length of the segment, in coordinates
+  float *qin;
+  const float *tin, *pin;  // the segment's target and momenta
+};
+
+__global__ void __launch_bounds__(256) k_badmit(AdmitArgs a) {
+  const int step = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
+  const int recs = a.slots + 2, rows = recs + kNumVecs + 2 * a.m + 1;
+  for (int row = blockIdx.y; row < rows; row += gridDim.y) {
+    const int v = row - recs, h = v - kNumVecs;
+    if (v < 0) {
+      float4* r = (row < a.slots ? a.traj + row * a.slot : a.adj + (row - a.slots) * a.slot) + a.r0;
+      for (size_t i = t0; i < a.rl; i += step) r[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if (h < 0) {
+      double* d = a.vec[v] + a.b3;
+      const float* src = v == 0 ? a.pin : v == 1 ? a.tin : nullptr;
+      for (int i = t0; i < a.e3; i += step) d[i] = src && i < a.n3 ? static_cast<double>(src[i]) : 0.0;
+    } else if (h < 2 * a.m) {
+      double* d = (h < a.m ? a.S + h * a.stride : a.Y + (h - a.m) * a.stride) + a.b3;
+      for (int i = t0; i < a.e3; i += step) d[i] = 0.0;
+    } else {
+      for (int i = a.n3 + t0; i < a.e3; i += step) a.qin[a.b3 + i] = 0.f;
+    }
+  }
+}
 
 // q64 <- q0 (packed FP32 input), p64 <- x, record slot 0, for listed problems.
 __global__ void __launch_bounds__(kBT) k_bpack(const int* list, const BatchProb* probs, const float* qin,
@@ -408,56 +451,62 @@ struct BatchEngine {
     // items: one per target tile of every problem, for the smaller of the
     // two kinds' tile sizes
     max_items = cap / std::min(fcfg.threads, bcfg.threads) + max_probs;
-    auto get = [&](void** p, size_t b) -> cudaError_t {
-      cudaError_t e = cudaMalloc(p, b + 256);
-      if (e == cudaSuccess) {
-        allocs.push_back(*p);
-        bytes += b;
+    // One device and one pinned allocation, carved up: an allocation each took
+    // 25 us, 33 of them 0.8 ms, and their release as much again.
+    std::vector<std::pair<void**, size_t>> want;
+    const auto get = [&](void** p, size_t b) { want.push_back({p, (b + 511) / 256 * 256}); };
+    const auto carve = [&](void* base) {
+      char* c = static_cast<char*>(base);
+      for (auto& x : want) {
+        *x.first = c;
+        c += x.second;
       }
-      return e;
+      want.clear();
+    };
+    const auto total = [&] {
+      size_t b = 0;
+      for (auto& x : want) b += x.second;
+      return b;
     };
     const size_t c3 = 3 * static_cast<size_t>(cap), slot = static_cast<size_t>(kRecF4) * (cap / 2);
-    GS_CUDA(get((void**)&traj, sizeof(float4) * slot * (T + 1)));
-    GS_CUDA(get((void**)&adj, sizeof(float4) * slot * 2));
+    get((void**)&traj, sizeof(float4) * slot * (T + 1));
+    get((void**)&adj, sizeof(float4) * slot * 2);
     for (double** p : {&q64, &p64, &a64, &b64, &t64, &hp0, &hq0, &gp64, &x, &g, &d, &xt, &gt})
-      GS_CUDA(get((void**)p, sizeof(double) * c3));
-    GS_CUDA(get((void**)&S, sizeof(double) * c3 * m));
-    GS_CUDA(get((void**)&Y, sizeof(double) * c3 * m));
-    GS_CUDA(get((void**)&qin, sizeof(float) * c3));
-    GS_CUDA(get((void**)&red_h, sizeof(double) * static_cast<size_t>(max_items) * 16));
-    GS_CUDA(get((void**)&red_m, sizeof(double) * static_cast<size_t>(max_items) * 16));
-    GS_CUDA(get((void**)&probs_d, sizeof(BatchProb) * max_probs));
-    GS_CUDA(get((void**)&items_d, sizeof(BatchItem) * 2 * static_cast<size_t>(max_items)));
-    for (int** p : {&list_d, &item0_d, &ntiles_d, &slot_d}) GS_CUDA(get((void**)p, sizeof(int) * max_probs));
-    GS_CUDA(get((void**)&loss_d, sizeof(double) * max_probs));
-    GS_CUDA(get((void**)&dots_d, sizeof(double) * 4 * max_probs));
-    GS_CUDA(get((void**)&a_d, sizeof(double) * max_probs));
-    GS_CUDA(get((void**)&alpha_d, sizeof(double) * kMaxM * max_probs));
-    GS_CUDA(get((void**)&dist_d, sizeof(double) * 2 * max_probs));
-    GS_CUDA(get((void**)&state_d, sizeof(TwoLoopState) * max_probs));
-    GS_CUDA(get((void**)&status_d, sizeof(unsigned) * 8));
+      get((void**)p, sizeof(double) * c3);
+    get((void**)&S, sizeof(double) * c3 * m);
+    get((void**)&Y, sizeof(double) * c3 * m);
+    get((void**)&qin, sizeof(float) * c3);
+    get((void**)&red_h, sizeof(double) * static_cast<size_t>(max_items) * 16);
+    get((void**)&red_m, sizeof(double) * static_cast<size_t>(max_items) * 16);
+    get((void**)&probs_d, sizeof(BatchProb) * max_probs);
+    get((void**)&items_d, sizeof(BatchItem) * 2 * static_cast<size_t>(max_items));
+    for (int** p : {&list_d, &item0_d, &ntiles_d, &slot_d}) get((void**)p, sizeof(int) * max_probs);
+    get((void**)&loss_d, sizeof(double) * max_probs);
+    get((void**)&dots_d, sizeof(double) * 4 * max_probs);
+    get((void**)&a_d, sizeof(double) * max_probs);
+    get((void**)&alpha_d, sizeof(double) * kMaxM * max_probs);
+    get((void**)&dist_d, sizeof(double) * 2 * max_probs);
+    get((void**)&state_d, sizeof(TwoLoopState) * max_probs);
+    get((void**)&status_d, sizeof(unsigned) * 8);
+    bytes = total();
+    void* base = nullptr;
+    GS_CUDA(cudaMalloc(&base, bytes));
+    allocs.push_back(base);
+    carve(base);
     GS_CUDA(cudaMemset(status_d, 0, sizeof(unsigned) * 8));
-    auto host = [&](void** p, size_t b) -> cudaError_t {
-      cudaError_t e = cudaMallocHost(p, b);
-      if (e == cudaSuccess) pinned.push_back(*p);
-      return e;
-    };
-    GS_CUDA(host((void**)&items_h, sizeof(BatchItem) * 2 * static_cast<size_t>(max_items)));
-    for (int** p : {&item0_h, &ntiles_h, &slot_h}) GS_CUDA(host((void**)p, sizeof(int) * max_probs));
-    GS_CUDA(host((void**)&lists_h, sizeof(int) * static_cast<size_t>(max_probs) * kListRing));
-    GS_CUDA(host((void**)&stv_h, sizeof(TwoLoopState) * max_probs));
-    GS_CUDA(host((void**)&ah_h, sizeof(double) * max_probs));
-    GS_CUDA(host((void**)&loss_h, sizeof(double) * max_probs));
-    GS_CUDA(host((void**)&dots_h, sizeof(double) * 4 * max_probs));
-    GS_CUDA(host((void**)&status_h, sizeof(unsigned) * 8));
-    // every optimiser vector starts at zero (never read before written, but
-    // a stale NaN must not be able to leak through a zero coefficient)
-    for (double* p : {x, g, d, xt, gt, q64, p64, a64, b64, t64, hp0, hq0, gp64})
-      GS_CUDA(cudaMemset(p, 0, sizeof(double) * c3));
-    GS_CUDA(cudaMemset(S, 0, sizeof(double) * c3 * m));
-    GS_CUDA(cudaMemset(Y, 0, sizeof(double) * c3 * m));
-    GS_CUDA(cudaMemset(traj, 0, sizeof(float4) * slot * (T + 1)));
-    GS_CUDA(cudaMemset(adj, 0, sizeof(float4) * slot * 2));
+    get((void**)&items_h, sizeof(BatchItem) * 2 * static_cast<size_t>(max_items));
+    for (int** p : {&item0_h, &ntiles_h, &slot_h}) get((void**)p, sizeof(int) * max_probs);
+    get((void**)&lists_h, sizeof(int) * static_cast<size_t>(max_probs) * kListRing);
+    get((void**)&stv_h, sizeof(TwoLoopState) * max_probs);
+    get((void**)&ah_h, sizeof(double) * max_probs);
+    get((void**)&loss_h, sizeof(double) * max_probs);
+    get((void**)&dots_h, sizeof(double) * 4 * max_probs);
+    get((void**)&status_h, sizeof(unsigned) * 8);
+    base = nullptr;
+    GS_CUDA(cudaMallocHost(&base, total()));
+    pinned.push_back(base);
+    carve(base);
+    // A problem's admission clears its segment of every array (k_badmit).
     probs_h.assign(max_probs, BatchProb{});
     slots.assign(max_probs, Problem{});
     for (int i = max_probs - 1; i >= 0; --i) free_slots.push_back(i);
@@ -545,60 +594,59 @@ struct BatchEngine {
       }
     }
     const size_t n3 = 3 * static_cast<size_t>(p.n), b3 = 3 * static_cast<size_t>(off);
-    // A reused segment holds the previous problem's values.  Record padding
-    // must be exactly zero, and the new problem starts from a clean state:
-    // clear the segment in every record slot and every per-landmark array.
-    {
-      const size_t slot = static_cast<size_t>(kRecF4) * (cap / 2);
-      const size_t r0 = static_cast<size_t>(kRecF4) * (off / 2), rl = static_cast<size_t>(kRecF4) * (npad / 2);
-      cudaError_t e0 = cudaSuccess;
-      for (int k = 0; k <= T && e0 == cudaSuccess; ++k)
-        e0 = cudaMemsetAsync(traj + k * slot + r0, 0, rl * sizeof(float4), st);
-      for (int k = 0; k < 2 && e0 == cudaSuccess; ++k) e0 = cudaMemsetAsync(adj + k * slot + r0, 0, rl * sizeof(float4), st);
-      const size_t e3 = 3 * static_cast<size_t>(npad);
-      for (double* arr : {q64, p64, a64, b64, t64, hp0, hq0, gp64, x, g, d, xt, gt})
-        if (e0 == cudaSuccess) e0 = cudaMemsetAsync(arr + b3, 0, e3 * sizeof(double), st);
-      for (int j = 0; j < m && e0 == cudaSuccess; ++j) {
-        e0 = cudaMemsetAsync(S + j * stride() + b3, 0, e3 * sizeof(double), st);
-        if (e0 == cudaSuccess) e0 = cudaMemsetAsync(Y + j * stride() + b3, 0, e3 * sizeof(double), st);
+    // Inputs: q0, target and p0 as FP32, then one kernel converts them and
+    // clears the rest of the segment.  Host arrays go up as they are.
+    const float* in[3] = {q0, target, p0};
+    const float* hv[3] = {q0, target, p0};  // what the host can read
+    float* const up[3] = {qin + b3, reinterpret_cast<float*>(gt + b3), reinterpret_cast<float*>(xt + b3)};
+    std::vector<float> copy[3];
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
+      if (!in[k]) {
+        e = cudaMemsetAsync(up[k], 0, n3 * sizeof(float), st);
+        continue;
       }
-      if (e0 == cudaSuccess) e0 = cudaMemsetAsync(qin + b3, 0, e3 * sizeof(float), st);
-      if (e0 != cudaSuccess) {
-        *err = fail(GS_ECUDA, std::string("clearing a segment: ") + cudaGetErrorString(e0));
-        retire(sl);
-        return -1;
+      if (pointer_kind(in[k]) != kPtrHost) {
+        copy[k].resize(n3);
+        hv[k] = copy[k].data();
+        e = cudaMemcpy(copy[k].data(), in[k], n3 * sizeof(float), cudaMemcpyDefault);
       }
+      if (e == cudaSuccess) e = cudaMemcpyAsync(up[k], hv[k], n3 * sizeof(float), cudaMemcpyHostToDevice, st);
     }
-    // Inputs: q0 -> qin (FP32), target -> t64, p0 -> x (FP64); padding zero.
-    std::vector<double> tmp(3 * static_cast<size_t>(npad), 0.0);
-    std::vector<float> tq(3 * static_cast<size_t>(npad), 0.f);
-    auto fetch = [&](const float* src, float* dst) -> cudaError_t {
-      if (!src) {
-        std::fill(dst, dst + n3, 0.f);
-        return cudaSuccess;
-      }
-      return cudaMemcpy(dst, src, n3 * sizeof(float), cudaMemcpyDefault);
-    };
-    cudaError_t e = fetch(q0, tq.data());
-    if (e == cudaSuccess) e = cudaMemcpyAsync(qin + b3, tq.data(), tq.size() * sizeof(float), cudaMemcpyHostToDevice, st);
-    std::vector<float> tt(3 * static_cast<size_t>(npad), 0.f);
-    if (e == cudaSuccess) e = fetch(target, tt.data());
-    for (size_t i = 0; i < tt.size(); ++i) tmp[i] = tt[i];
-    if (e == cudaSuccess) e = cudaMemcpyAsync(t64 + b3, tmp.data(), tmp.size() * sizeof(double), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    std::vector<float> tp(3 * static_cast<size_t>(npad), 0.f);
-    if (e == cudaSuccess) e = fetch(p0, tp.data());
-    for (size_t i = 0; i < tp.size(); ++i) tmp[i] = tp[i];
-    if (e == cudaSuccess) e = cudaMemcpyAsync(x + b3, tmp.data(), tmp.size() * sizeof(double), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) {
+      AdmitArgs ad{};
+      ad.traj = traj;
+      ad.adj = adj;
+      ad.slot = static_cast<size_t>(kRecF4) * (cap / 2);
+      ad.r0 = static_cast<size_t>(kRecF4) * (off / 2);
+      ad.rl = static_cast<size_t>(kRecF4) * (npad / 2);
+      ad.slots = T + 1;
+      double* const vecs[kNumVecs] = {x, t64, q64, p64, a64, b64, hp0, hq0, gp64, g, d};
+      std::copy(vecs, vecs + kNumVecs, ad.vec);
+      ad.S = S;
+      ad.Y = Y;
+      ad.stride = stride();
+      ad.b3 = b3;
+      ad.m = m;
+      ad.n3 = static_cast<int>(n3);
+      ad.e3 = 3 * npad;
+      ad.qin = qin;
+      ad.tin = up[1];
+      ad.pin = up[2];
+      const int rows = ad.slots + 2 + kNumVecs + 2 * m + 1;
+      k_badmit<<<dim3(std::min((ad.e3 + 1023) / 1024, 64), std::min(rows, 4096)), 256, 0, st>>>(ad);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the caller's arrays are free again
     if (e != cudaSuccess) {
       *err = fail(GS_ECUDA, std::string("staging a problem: ") + cudaGetErrorString(e));
       retire(sl);
       return -1;
     }
     bool finite = true;
-    for (size_t i = 0; i < n3; ++i)
-      if (!std::isfinite(tq[i]) || !std::isfinite(tt[i]) || !std::isfinite(tp[i])) finite = false;
+    for (int k = 0; k < 3; ++k)
+      for (size_t i = 0; hv[k] && i < n3; ++i)
+        if (!std::isfinite(hv[k][i])) finite = false;
     if (!finite) {  // reported as failed by the next round, never evaluated
       p.phase = kDone;
       p.status = -1;
