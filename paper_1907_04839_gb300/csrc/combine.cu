@@ -104,22 +104,27 @@ __global__ void __launch_bounds__(kThreads) k_partials_to_out(const Partial* par
   else out_b[3 * i + k] = (float)ds_to_double(acc[3 + k]);
 }
 
-// One thread per landmark slot i < npad (padding written as zeros).
-__global__ void __launch_bounds__(kThreads) k_to_records(const float* x, const float* y, float4* rec, int n, int npad,
-                                                         double sx, double sy, int ab_layout, unsigned* status) {
+// One thread per landmark slot i < npad (padding written as zeros);
+// blockIdx.y picks the record set.
+struct RecordSets {
+  RecordSet set[2];
+};
+
+__global__ void __launch_bounds__(kThreads) k_to_records(RecordSets sets, int n, int npad, unsigned* status) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= npad) return;
-  float* r = reinterpret_cast<float*>(rec + (i >> 1) * kRecF4) + (i & 1);
-  const float fx = ab_layout ? 1.f : -1.f, fy = ab_layout ? -1.f : 1.f;
+  const RecordSet& s = sets.set[blockIdx.y];
+  float* r = reinterpret_cast<float*>(s.rec + (i >> 1) * kRecF4) + (i & 1);
+  const float fx = s.ab_layout ? 1.f : -1.f, fy = s.ab_layout ? -1.f : 1.f;
   for (int k = 0; k < 3; ++k) {
     float a = 0.f, b = 0.f;
     if (i < n) {
-      a = x[3 * i + k];
-      b = y[3 * i + k];
+      a = s.a[3 * i + k];
+      b = s.b[3 * i + k];
       if (!isfinite(a) || !isfinite(b)) atomicOr(status, kErrNonFinite);
     }
-    r[2 * k] = fx * (float)(sx * a);
-    r[6 + 2 * k] = fy * (float)(sy * b);
+    r[2 * k] = fx * (float)(s.sa * a);
+    r[6 + 2 * k] = fy * (float)(s.sb * b);
   }
 }
 
@@ -182,9 +187,10 @@ cudaError_t launch_partials_to_out(const Partial* part, int splits, int n, int n
   return cudaGetLastError();
 }
 
-cudaError_t launch_to_records(const float* a, const float* b, float4* rec, int n, int npad, double sa, double sb,
-                              int ab_layout, unsigned* status, cudaStream_t st) {
-  k_to_records<<<blocks_for(npad), kThreads, 0, st>>>(a, b, rec, n, npad, sa, sb, ab_layout, status);
+cudaError_t launch_to_records(const RecordSet* sets, int count, int n, int npad, unsigned* status, cudaStream_t st) {
+  RecordSets r{};
+  for (int k = 0; k < count; ++k) r.set[k] = sets[k];
+  k_to_records<<<dim3(blocks_for(npad), count), kThreads, 0, st>>>(r, n, npad, status);
   return cudaGetLastError();
 }
 

@@ -578,8 +578,9 @@ gs_status run_step(int kind, int64_t N, double sigma, const float* q, const floa
   gs_status s = get_workspace(&w);
   if (s != GS_OK) return s;
   const int n = static_cast<int>(N), npad = round_up(n, kPad);
-  const PairConfig c = kind == 0 ? choose_forward_config(npad, w->num_sms) : choose_backward_config(npad, w->num_sms);
-  if ((s = reserve(*w, npad, 1, c.splits)) != GS_OK) return s;
+  const StepConfig c = choose_step_config(kind, npad, w->num_sms);
+  if (c.threads == 0) return fail(GS_EINVAL, "no step kernel configuration");
+  if ((s = reserve(*w, npad, 1, 1)) != GS_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t n3 = 3 * static_cast<size_t>(n);
   bool host = false;
@@ -590,41 +591,31 @@ gs_status run_step(int kind, int64_t N, double sigma, const float* q, const floa
     if ((s = stage_in(alpha, w->in_a, n3, st, &da, &host)) != GS_OK) return s;
     if ((s = stage_in(beta, w->in_t, n3, st, &db, &host)) != GS_OK) return s;
   }
+  // Hp, Hq / dalpha, dbeta straight from a dry step of the fused kernels: the
+  // records, then the pair sums with their cluster reduction.
+  float *o0 = nullptr, *o1 = nullptr;
+  if ((s = out_ptr(out0, w->out_a, &o0)) != GS_OK) return s;
+  if ((s = out_ptr(out1, w->out_b, &o1)) != GS_OK) return s;
   const KernelScales sc = make_scales(sigma);
-  GS_CUDA(launch_to_records(dq, dp, w->traj, n, npad, sc.kq, 1.0, 0, w->status, st));
-  if (kind == 0) {
-    PairFwdArgs a;
-    a.qp = w->traj;
-    a.part = w->part;
-    a.npad = npad;
-    a.split_len = c.split_len;
-    a.kappa = static_cast<float>(sc.kappa);
-    a.status = w->status;
-    GS_CUDA(launch_pair_forward(c, a, st, false));
-  } else {
-    GS_CUDA(launch_to_records(da, db, w->adj, n, npad, 1.0, sc.kappa, 1, w->status, st));
-    PairBwdArgs a;
-    a.qp = w->traj;
-    a.ab = w->adj;
-    a.part = w->part;
-    a.npad = npad;
-    a.split_len = c.split_len;
-    a.kq = static_cast<float>(sc.kq);
-    a.kappa = static_cast<float>(sc.kappa);
-    a.status = w->status;
-    GS_CUDA(launch_pair_backward(c, a, st, false));
-  }
-  // Partials hold (Hp, Hq) forward and (dalpha, dbeta) backward.
-  GS_CUDA(launch_partials_to_out(w->part, c.splits, n, npad, w->out_a, w->out_b, st));
+  const RecordSet sets[2] = {{dq, dp, w->traj, sc.kq, 1.0, 0}, {da, db, w->adj, 1.0, sc.kappa, 1}};
+  GS_CUDA(launch_to_records(sets, kind + 1, n, npad, w->status, st));
   w->clean_n = -1;  // traj slot 0 / adjoint arrays were overwritten
-  bool want_sync = host;
   if (kind == 0) {
-    if ((s = copy_out(out1, w->out_a, n3, st, &want_sync)) != GS_OK) return s;  // Hp
-    if ((s = copy_out(out0, w->out_b, n3, st, &want_sync)) != GS_OK) return s;  // Hq
+    StepFwdArgs a = forward_step_args(*w, c, 0, n, 1, 0, sigma, 0.0);
+    a.dry = 1;
+    a.out_q = o0;
+    a.out_p = o1;
+    GS_CUDA(launch_step_forward(c, a, st, true));
   } else {
-    if ((s = copy_out(out0, w->out_a, n3, st, &want_sync)) != GS_OK) return s;  // dalpha
-    if ((s = copy_out(out1, w->out_b, n3, st, &want_sync)) != GS_OK) return s;  // dbeta
+    StepBwdArgs b = backward_step_args(*w, c, n, 1, 0, sigma);
+    b.dry = 1;
+    b.out_a = o0;
+    b.out_b = o1;
+    GS_CUDA(launch_step_backward(c, b, st, true));
   }
+  bool want_sync = host;
+  if (o0 != out0 && (s = copy_out(out0, o0, n3, st, &want_sync)) != GS_OK) return s;
+  if (o1 != out1 && (s = copy_out(out1, o1, n3, st, &want_sync)) != GS_OK) return s;
   if (want_sync) return finish_sync(*w, st);
   return GS_OK;
 }
@@ -716,8 +707,8 @@ gs_status time_pair_config(int kind_in, int64_t N, double sigma, const float* q,
     if ((s = stage_in(beta, w->in_t, n3, st, &db, &host)) != GS_OK) return s;
   }
   const KernelScales ks = make_scales(sigma);
-  GS_CUDA(launch_to_records(dq, dp, w->traj, n, npad, ks.kq, 1.0, 0, w->status, st));
-  if (bwd) GS_CUDA(launch_to_records(da, db, w->adj, n, npad, 1.0, ks.kappa, 1, w->status, st));
+  const RecordSet sets[2] = {{dq, dp, w->traj, ks.kq, 1.0, 0}, {da, db, w->adj, 1.0, ks.kappa, 1}};
+  GS_CUDA(launch_to_records(sets, bwd ? 2 : 1, n, npad, w->status, st));
   w->clean_n = -1;
   PairFwdArgs fa;
   fa.qp = w->traj;

@@ -142,7 +142,8 @@ struct StepFwdArgs {
   double* red_m;
   unsigned* ticket;
   double* scalars;     // [0] = H0, [1] = loss, [2] = H at the end state (terminal launch)
-  int dry;             // tuning: compute everything, write nothing
+  int dry;             // compute everything, touch no state (timing; the one-step entry points)
+  float *out_q, *out_p;  // dry: where Hq and Hp go as (N, dim) arrays (null: nowhere)
   unsigned* status;
   // Variants (all zero: an Euler step, the kinetic term at t = 0).
   int rk;              // 1: stage `stage` (0..3) of an RK4 step
@@ -175,6 +176,7 @@ struct StepBwdArgs {
   float* grad_q0;
   double* grad_p0_64;  // FP64 copy of dL/dp0 (may be null)
   int dry;
+  float *out_a, *out_b;  // dry: where dalpha and dbeta go (null: nowhere)
   unsigned* status;
   // Variants (all zero: a reverse Euler step, gradient with the H(p0, q0) term).
   int rk;              // 1: stage `stage` (3..0) of the reverse of an RK4 step; the
@@ -326,8 +328,14 @@ cudaError_t launch_partials_to_out(const Partial* part, int splits, int n, int n
                                    float* out_a, float* out_b, cudaStream_t st);
 // Two (N,3) float32 arrays -> pair records {-sa * a, sb * b} (QP: a = q,
 // b = p) or {sa * a, -sb * b} (AB: a = alpha, b = beta), zero-padded to npad.
-cudaError_t launch_to_records(const float* a, const float* b, float4* rec, int n, int npad, double sa, double sb,
-                              int ab_layout, unsigned* status, cudaStream_t st);
+struct RecordSet {
+  const float *a, *b;
+  float4* rec;
+  double sa, sb;
+  int ab_layout;
+};
+// One or two sets of n landmarks in one launch.
+cudaError_t launch_to_records(const RecordSet* sets, int count, int n, int npad, unsigned* status, cudaStream_t st);
 
 int combine_threads();
 int combine_group();  // lanes per landmark in the combine kernels

@@ -129,7 +129,8 @@ extern "C" gs_status step_forward_noalloc(int64_t N, double sigma, const float* 
   // records (padding included) and the partials are fully rewritten below.
   cudaError_t e = cudaMemsetAsync(status, 0, 4 * sizeof(unsigned), st);
   if (e != cudaSuccess) return cuda_fail(e);
-  if ((e = launch_to_records(q, p, qp, n, npad, sc.kq, 1.0, 0, status, st)) != cudaSuccess) return cuda_fail(e);
+  const RecordSet set{q, p, qp, sc.kq, 1.0, 0};
+  if ((e = launch_to_records(&set, 1, n, npad, status, st)) != cudaSuccess) return cuda_fail(e);
   PairFwdArgs a;
   a.qp = qp;
   a.part = part;

@@ -260,7 +260,11 @@ __device__ __forceinline__ void forward_body(const StepFwdArgs& a, const StepVie
           y = rp[D + k];
         },
         Hp, Hq);
-    if (a.dry) {  // timing only: keep the reduction, touch no state
+    if (a.dry) {  // keep the reduction, touch no state
+      if (a.out_q) {
+        a.out_q[D * i + k] = (float)Hq;
+        a.out_p[D * i + k] = (float)Hp;
+      }
       hc += Hp + Hq;
       continue;
     }
@@ -434,7 +438,12 @@ __device__ __forceinline__ void backward_body(const StepBwdArgs& a, const StepVi
           dA, dB);
     }
     if (a.dry) {
-      if (!isfinite(dA + dB)) atomicOr(a.status, kErrNonFinite);
+      if (a.out_a) {
+        a.out_a[D * i + k] = (float)dA;
+        a.out_b[D * i + k] = (float)dB;
+      } else if (!isfinite(dA + dB)) {
+        atomicOr(a.status, kErrNonFinite);
+      }
       continue;
     }
     const int tt = D * i + k;

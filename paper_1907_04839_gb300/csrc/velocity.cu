@@ -286,7 +286,8 @@ extern "C" gs_status velocity_field(int64_t N, int64_t M, double sigma, const fl
   if ((s = stage_in(p, w->in_p, n3, st, &dp, &host)) != GS_OK) return s;
   if ((s = stage_in(x, w->pts_in, m3, st, &dx, &host)) != GS_OK) return s;
   const KernelScales sc = make_scales(sigma);
-  GS_CUDA(launch_to_records(dq, dp, w->traj, n, npad, sc.kq, 1.0, 0, w->status, st));
+  const RecordSet qp{dq, dp, w->traj, sc.kq, 1.0, 0};
+  GS_CUDA(launch_to_records(&qp, 1, n, npad, w->status, st));
   w->clean_n = -1;  // record slot 0 was overwritten
   k_points_to64<<<conv_blocks(m3), 256, 0, st>>>(dx, w->pts64, m3);
   GS_CUDA(cudaGetLastError());
