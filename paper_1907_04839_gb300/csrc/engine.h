@@ -36,9 +36,10 @@ struct GraphKey {
   int integ = 0;  // GS_EULER or GS_RK4
   int h_end = 0;  // the loss takes the kinetic term at t = 1
   int dim = 3;    // 3-D or planar landmarks
+  int ordered = 0;  // landmarks packed in spatial order, culling step kernels
   bool operator<(const GraphKey& o) const {
-    return std::tie(kind, n, T, sigma, lambda, ckpt, timed, integ, h_end, dim) <
-           std::tie(o.kind, o.n, o.T, o.sigma, o.lambda, o.ckpt, o.timed, o.integ, o.h_end, o.dim);
+    return std::tie(kind, n, T, sigma, lambda, ckpt, timed, integ, h_end, dim, ordered) <
+           std::tie(o.kind, o.n, o.T, o.sigma, o.lambda, o.ckpt, o.timed, o.integ, o.h_end, o.dim, o.ordered);
   }
 };
 
@@ -108,6 +109,14 @@ struct Workspace {
   bool phase_timing = false;
   cudaEvent_t phase[3] = {nullptr, nullptr, nullptr};
   LbfgsBufs lb;
+  // Spatial order (order.cu; grown on demand): the caller's index of each
+  // landmark, the codes it was ordered by, the dense flag, and the boxes of the runs of every
+  // state of a sweep.
+  int cap_ord = 0;
+  size_t cap_box = 0;
+  std::vector<void*> ord_allocs;
+  int *perm = nullptr, *dense = nullptr;
+  unsigned *codes = nullptr, *boxes = nullptr;
   // Query points of velocity_field / flow_points (grown on demand).
   int cap_pts = 0;
   std::vector<void*> pt_allocs;
@@ -126,6 +135,10 @@ struct Workspace {
     for (void* p : pt_allocs) cudaFree(p);
     pt_allocs.clear();
     cap_pts = 0;
+    for (void* p : ord_allocs) cudaFree(p);
+    ord_allocs.clear();
+    cap_ord = 0;
+    cap_box = 0;
     cap_npad = cap_T = cap_splits = cap_red = cap_ck = 0;
     clean_n = -1;
   }
@@ -153,6 +166,12 @@ gs_status get_graph(Workspace& w, const GraphKey& key, cudaGraphExec_t* out);
 // trajectory is at most a few MB).
 bool small_path(const Workspace& w, const gs_params& prm);
 int shoot_ckpt(const Workspace& w, const gs_params& prm);
+// Whether a sweep of J evaluations packs its landmarks in spatial order
+// (order.cu); the words of the boxes of one state; room for the order
+// of npad landmarks and nbox words of boxes.
+bool use_order(int npad, int J, int dim);
+size_t box_words(int npad);
+gs_status reserve_order(Workspace& w, int npad, size_t nbox);
 // Device destinations of a sweep's results; null: not wanted.
 struct ShootOut {
   float *a = nullptr, *b = nullptr;  // kind 0: q(1), p(1); kind 1: dL/dp0, dL/dq0

@@ -91,6 +91,73 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // their pair sums, when the host asks for it (one-wave grids).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// ---------------------------------------------------------------- boxes of landmark runs
+// A run of kGran landmarks has kBoxWords words: [k] and [4 + k] hold the
+// largest v_k and the largest -v_k of the run's record positions v, as
+// integers in the order of the floats.  0 marks a run without landmarks, so
+// boxes start as zeros and grow by atomicMax (the order does not matter).
+__device__ __forceinline__ unsigned float_order(float f) {
+  const unsigned u = __float_as_uint(f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+__device__ __forceinline__ float order_float(unsigned e) {
+  return __uint_as_float((e & 0x80000000u) ? (e & 0x7fffffffu) : ~e);
+}
+
+__device__ __forceinline__ void box_add(unsigned* boxes, int i, int k, float v) {
+  unsigned* b = boxes + static_cast<size_t>(i / kGran) * kBoxWords + k;
+  atomicMax(b, float_order(v));
+  atomicMax(b + 4, float_order(-v));
+}
+
+// A box in record positions: largest v and largest -v per coordinate.
+template <int D>
+struct RunBox {
+  float hi[D], lo[D];  // lo: largest -v
+};
+
+// The words of one run's box, as loaded.
+struct BoxWords {
+  uint4 h, l;
+};
+
+__device__ __forceinline__ BoxWords load_box(const unsigned* boxes, int run) {
+  const uint4* p = reinterpret_cast<const uint4*>(boxes + static_cast<size_t>(run) * kBoxWords);
+  return BoxWords{__ldcg(p), __ldcg(p + 1)};
+}
+
+// The box; one without landmarks is out of everything's reach.
+template <int D>
+__device__ __forceinline__ RunBox<D> run_box(const BoxWords& w) {
+  const unsigned hh[3] = {w.h.x, w.h.y, w.h.z}, ll[3] = {w.l.x, w.l.y, w.l.z};
+  RunBox<D> b;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    b.hi[k] = w.h.x ? order_float(hh[k]) : -INFINITY;
+    b.lo[k] = w.h.x ? order_float(ll[k]) : -INFINITY;
+  }
+  return b;
+}
+
+// Squared prescaled distance from which a pair's Gaussian is exactly zero:
+// ex2 flushes results below 2^-126; one more unit covers the rounding of the
+// pair's own r2 and of the boxes' gap.
+constexpr float kReach2 = 127.f;
+
+// Whether boxes t and b have a pair in reach.
+template <int D>
+__device__ __forceinline__ bool in_reach(const RunBox<D>& t, const RunBox<D>& b) {
+  float r2 = 0.f;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    // distance between the intervals [-lo, hi]
+    const float gap = fmaxf(fmaxf(-t.lo[k] - b.hi[k], -b.lo[k] - t.hi[k]), 0.f);
+    r2 = fmaf(gap, gap, r2);
+  }
+  return !(r2 > kReach2);
+}
+
 // 2^x on the MUFU unit (flushes subnormal results to zero).
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;

@@ -31,6 +31,11 @@ enum : unsigned {
 constexpr int kPad = 64;      // landmark padding granule
 constexpr int kChunk = 128;   // sources staged in shared memory per bulk copy
 constexpr int kStages = 4;    // chunk buffers in flight per CTA
+constexpr int kGran = 32;     // landmarks per bounded run (order.cu)
+constexpr int kBoxWords = 8;  // words per run's box
+// Padded landmarks from which sweeps order them (3-D, planar), see order.cu.
+constexpr int kOrderNpad = 4608;
+constexpr int kOrderNpad2 = 3584;
 constexpr int kRecF4 = 3;     // float4 per pair record (two landmarks)
 constexpr int kRecBytes = 48;
 
@@ -117,6 +122,7 @@ struct StepConfig {
   int split_len;  // sources per CTA (multiple of 8)
   int policy;     // cluster scheduling: 0 driver default, 1 spread, 2 load balancing
   int groups;     // warp groups per CTA that split the CTA's sources (1: none)
+  bool cull;      // ordered landmarks: runs of sources out of a tile's reach are left out
 };
 
 struct StepFwdArgs {
@@ -158,6 +164,9 @@ struct StepFwdArgs {
                        // arrays); 0 or 3: 3-D
   int late_trigger;    // trigger the next launch after the pair sums (pdl_trigger)
   int combine64;       // add the split partials in FP64 (0: double-single)
+  const unsigned* box;  // culling kernels: boxes of the state's runs
+  const int* dense;     // and whether nearly all pairs are in reach (order.cu)
+  unsigned* box_next;   // boxes of the state written (null: they stand already)
 };
 
 struct StepBwdArgs {
@@ -189,6 +198,9 @@ struct StepBwdArgs {
   int dim;             // 2: planar landmarks; 0 or 3: 3-D
   int late_trigger;    // trigger the next launch after the pair sums (pdl_trigger)
   int combine64;       // add the split partials in FP64 (0: double-single)
+  const unsigned* box;  // culling kernels: boxes of the state's runs
+  const int* dense;     // and whether nearly all pairs are in reach (order.cu)
+  const int* perm;      // the caller's index of each landmark (null: its own)
 };
 
 // Packed batches of independent problems.  Problem b occupies landmarks
@@ -309,6 +321,7 @@ struct PackArgs {
   double kq;
   unsigned* status;
   int dim;             // 2: planar landmarks ((N,2) arrays); 0 or 3: 3-D
+  int npad;            // launch_order_pack: the padding of the slot is zeroed too
 };
 
 struct UnpackArgs {
@@ -319,6 +332,14 @@ struct UnpackArgs {
 
 cudaError_t launch_pack(const PackArgs& a, cudaStream_t st);
 cudaError_t launch_unpack(const UnpackArgs& a, cudaStream_t st);
+// Pack in spatial order (order.cu): perm[r] is the caller's index of landmark
+// r; codes is scratch (n rounded up to 32); boxes[0, nbox) are zeroed and
+// the first set grown to the packed state.  dense[1] is set when nearly all
+// pairs are in reach; dense[0] is a ticket (zero between calls).
+cudaError_t launch_order_pack(const PackArgs& a, unsigned* codes, int* perm, unsigned* boxes, size_t nbox, int* dense,
+                              cudaStream_t st);
+// out[perm[r]] = x64[r] as float32.
+cudaError_t launch_unpack_perm(const double* x64, const int* perm, float* out, int n, int dim, cudaStream_t st);
 // Restore an FP64 state checkpoint into q64, p64 and record slot 0 of rec,
 // with the same rounding as the step kernels' epilogue.
 cudaError_t launch_restore(const double* ckq, const double* ckp, double* q64, double* p64, float4* rec, int n,

@@ -40,6 +40,7 @@ constexpr int kUnroll = 8;  // split lengths are multiples of this
 template <int NA, int D = 3>
 struct StageBuf {
   float4 buf[kStages][NA][D * kChunk / 2];
+  float4 ahead[4 * D];  // a loop that loads ahead may read (not use) this far past the last stage
 };
 
 // full[s]: the bulk copies of the chunk in stage s have landed (transaction
@@ -61,15 +62,16 @@ __device__ __forceinline__ void pipe_init(Pipe& p, int warps) {
   fence_mbar_init();
 }
 
-// Issue the bulk copies of chunk c (NA record arrays) into stage c % kStages.
+// Issue the bulk copies of chunk c (NA record arrays) into stage c % kStages (of
+// the absolute chunk number, where it differs).
 // Source offsets and lengths are even, so records are copied whole.
 template <int NA, int D>
 __device__ __forceinline__ void issue_chunk(StageBuf<NA, D>& st, Pipe& pp, const float4* const* src, int j0, int j1,
-                                            int c) {
+                                            int c, int abs = -1) {
   const int off = j0 + c * kChunk;
   const int len = min(kChunk, j1 - off);
   const unsigned bytes = static_cast<unsigned>(len) * (16 * D / 2);
-  const int s = c % kStages;
+  const int s = (abs < 0 ? c : abs) % kStages;
   uint64_t* bar = &pp.full[s];
   mbar_arrive_expect_tx(bar, NA * bytes);
 #pragma unroll
@@ -141,6 +143,174 @@ __device__ bool stream_sources(StageBuf<NA, D>& st, Pipe& pp, const float4* cons
   return true;
 }
 
+// Runs of a culling kernel's list per window: half a KB, so that the one-warp
+// reverse CTAs still fit eight to an SM (seven were 20 % slower at N = 8192).
+constexpr int kListCap = 128;
+constexpr int kGranPerChunk = kChunk / kGran;
+// Copy runs list[4c .. 4c+3] (fewer at the end of the list) of every record
+// array into the stage of absolute chunk `abs`.
+template <int NA, int D>
+__device__ __forceinline__ void issue_runs(StageBuf<NA, D>& st, Pipe& pp, const float4* const* src, const unsigned* list,
+                                           int cnt, int c, int abs) {
+  constexpr int kRunF4 = kGran / 2 * D;  // float4 per run and array
+  const int m = min(kGranPerChunk, cnt - c * kGranPerChunk);
+  const int s = abs % kStages;
+  uint64_t* bar = &pp.full[s];
+  mbar_arrive_expect_tx(bar, NA * m * kRunF4 * 16);
+  for (int g = 0; g < m; ++g) {
+    const size_t off = static_cast<size_t>(list[c * kGranPerChunk + g]) * kRunF4;
+#pragma unroll
+    for (int a = 0; a < NA; ++a) bulk_g2s(&st.buf[s][a][g * kRunF4], src[a] + off, kRunF4 * 16, bar);
+  }
+}
+
+// stream_sources over nsrc sources: those from first on, or (first < 0) the
+// runs of list.  base: chunks the CTA has streamed before (the stage ring and
+// its barrier phases run on); the caller adds the chunks of this call.  One
+// warp group.  One loop for both: two copies of it cost 17 registers and 8 % of
+// the forward step.
+template <int NA, int D, class Tile>
+__device__ bool stream_runs(StageBuf<NA, D>& st, Pipe& pp, const float4* const* src, const unsigned* list, int first,
+                            int nsrc, int base, Tile& tile, unsigned* status) {
+  const int tid = threadIdx.x;
+  const int nch = (nsrc + kChunk - 1) / kChunk;
+  const auto issue = [&](int c) {
+    if (first >= 0)
+      issue_chunk<NA, D>(st, pp, src, first, first + nsrc, c, base + c);
+    else
+      issue_runs<NA, D>(st, pp, src, list, nsrc / kGran, c, base + c);
+  };
+  int issued = 0;
+  if (tid == 0) {
+    for (; issued < nch && issued < kStages; ++issued) issue(issued);
+  }
+  volatile int* abort = &pp.abort;
+  for (int c = 0; c < nch; ++c) {
+    const int s = (base + c) % kStages;
+    const unsigned ph = ((base + c) / kStages) & 1;
+    if (*abort) break;
+    if (!mbar_wait(&pp.full[s], ph)) {
+      *abort = 1;
+      break;
+    }
+    const float4* bufs[NA];
+#pragma unroll
+    for (int a = 0; a < NA; ++a) bufs[a] = st.buf[s][a];
+    tile.consume(bufs, 0, min(kChunk, nsrc - c * kChunk));
+    __syncwarp();
+    if ((tid & 31) == 0) mbar_arrive(&pp.empty[s]);
+    if (tid == 0 && c + kStages < nch) {
+      if (mbar_wait(&pp.empty[s], ph)) {
+        fence_proxy_async_smem();
+        issue(c + kStages);
+        issued = c + kStages + 1;
+      } else {
+        *abort = 1;
+      }
+    }
+  }
+  __syncthreads();
+  if (*abort) {
+    if (tid == 0) {
+      atomicOr(status, kErrTimeout);
+      for (int d = max(0, issued - kStages); d < issued; ++d)
+        (void)mbar_wait(&pp.full[(base + d) % kStages], ((base + d) / kStages) & 1);
+    }
+    __syncthreads();
+    return false;
+  }
+  return true;
+}
+
+// Box of the M targets from tile0 on (whole runs; npad a multiple of a run).
+template <int D, int M>
+__device__ __forceinline__ RunBox<D> tile_box(const unsigned* boxes, int tile0, int nrun) {
+  static_assert(M % kGran == 0, "tiles are whole runs");
+  BoxWords w[M / kGran];
+#pragma unroll
+  for (int g = 0; g < M / kGran; ++g) w[g] = load_box(boxes, min(tile0 / kGran + g, nrun - 1));
+  RunBox<D> t = run_box<D>(w[0]);
+#pragma unroll
+  for (int g = 1; g < M / kGran; ++g) {
+    const RunBox<D> b = run_box<D>(w[g]);
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      t.hi[k] = fmaxf(t.hi[k], b.hi[k]);
+      t.lo[k] = fmaxf(t.lo[k], b.lo[k]);
+    }
+  }
+  return t;
+}
+
+// Runs [w0, w1) of CTA `rank` of C (its run m is run rank + m C): those in reach
+// of box tbox() go to list.  One warp, 32 runs at a time, in bit-reversed
+// order: neighbours on the curve land in different chunks, so that a target's
+// near sources, which carry its sum, do not all add up in one plain-FP32
+// sub-block.  Returns their count.
+template <int D, class Box>
+__device__ __forceinline__ int list_in_reach(const unsigned* boxes, Box tbox, int rank, int C, int w0, int w1,
+                                             unsigned* list) {
+  const unsigned lane = threadIdx.x & 31;
+  const int mine = static_cast<int>(__brev(lane) >> 27);
+  // the first boxes are on their way before the tile's are waited for
+  const auto at = [&](int m) { return rank + min(m + mine, w1 - 1) * C; };
+  BoxWords next = load_box(boxes, at(w0));
+  const RunBox<D> t = tbox();
+  int cnt = 0;
+  for (int m = w0; m < w1; m += 32) {
+    const RunBox<D> b = run_box<D>(next);
+    if (m + 32 < w1) next = load_box(boxes, at(m + 32));
+    const bool in = m + mine < w1 && in_reach(t, b);
+    const unsigned v = __ballot_sync(0xffffffffu, in);
+    if (in) list[cnt + __popc(v & ((1u << lane) - 1u))] = at(m);
+    cnt += __popc(v);
+  }
+  return cnt;
+}
+
+// The two uses, compiled apart from the pair loops: inlined, they cost the
+// loops up to 28 registers and, on a dense problem, 8 % of the forward step.
+template <int D, int M>
+__device__ __noinline__ int list_for_tile(const unsigned* boxes, int tile0, int nrun, int rank, int C, int w0, int w1,
+                                          unsigned* list) {
+  return list_in_reach<D>(boxes, [&] { return tile_box<D, M>(boxes, tile0, nrun); }, rank, C, w0, w1, list);
+}
+
+template <int D>
+__device__ __noinline__ int list_for_box(const unsigned* boxes, RunBox<D> t, int rank, int C, int w0, int w1,
+                                         unsigned* list) {
+  return list_in_reach<D>(boxes, [&] { return t; }, rank, C, w0, w1, list);
+}
+
+// The pair sums of a tile over every C-th run of the sources, from run `rank`
+// on, runs out of the tile's reach left out.  Interleaving gives the CTAs of
+// the cluster nearly equal lists, as neighbours on the curve are in or out of
+// reach together.  make(w0, w1, list) is
+// list_for_tile or list_for_box, called by warp 0.  list: kListCap + 1 words of
+// shared memory (the last holds the count).  dense: every source of [j0, j1)
+// instead.  Ends with a CTA barrier.
+template <int NA, int D, class Tile, class Make>
+__device__ __forceinline__ void sum_in_reach(StageBuf<NA, D>& st, Pipe& pp, const float4* const* src, Make make,
+                                             int nrun, int rank, int C, bool dense, int j0, int j1, Tile& tile,
+                                             unsigned* list, unsigned* status) {
+  const int mine = (nrun - rank + C - 1) / C;  // runs of this CTA
+  int base = 0, w0 = 0;
+  do {
+    int nsrc = j1 - j0;
+    if (!dense) {
+      if (threadIdx.x < 32) {
+        const int cnt = w0 < mine ? make(w0, min(w0 + kListCap, mine), list) : 0;
+        if (threadIdx.x == 0) list[kListCap] = cnt;
+      }
+      __syncthreads();
+      nsrc = static_cast<int>(list[kListCap]) * kGran;
+    }
+    if (!stream_runs<NA, D>(st, pp, src, list, dense ? j0 : -1, nsrc, base, tile, status)) return;
+    base += (nsrc + kChunk - 1) / kChunk;
+    w0 += kListCap;
+  } while (!dense && w0 < mine);
+}
+
 __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
@@ -170,6 +340,25 @@ __device__ __forceinline__ void rec_split(const float4* rec, float2 (&v)[2 * D])
     v[2 * f + 1] = hi2(x);
   }
 }
+
+// U records at p.
+template <int U, int D>
+__device__ __forceinline__ void load_records(const float4* p, float4 (&x)[U][D]) {
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int f = 0; f < D; ++f) x[u][f] = p[u * D + f];
+}
+
+// Records that the 64-thread reverse CTAs' loop loads ahead of the ones in use
+// where the grid has several waves (ordered sweeps, packed batches).  One warp's
+// loop alone on a scheduler takes 102.8 instead of 109.0 cycles a record; the
+// registers (96 to 119) decide what whole steps gain: 302 against 313 us at
+// N = 16384, 1533 against 1593 at 38785; 32-thread CTAs lose (94.2 against 90.2
+// at 8192), and so do one-wave grids (11.7 against 9.6 us at 1847, 29.5 against
+// 28.5 at 4096).  The forward loop gained nothing in whole gradients (four
+// ahead: 57.7 against 83.7 cycles alone, but 92 registers).
+constexpr int kAhead = 2;
 
 // One target against one source record (two sources) of StepForward.
 // q, p: the target, duplicated; v[k] = -q~_j, v[D + k] = p_j; aF += g p_j,
@@ -275,9 +464,7 @@ struct FwdTile {
           float2 v[2 * D];  // v[k] = -q~_j, v[D + k] = p_j
           rec_split<D>(Q + ((sb + jj) / 2 + u) * D, v);
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            fwd_record<D>(q[r], p[r], v, aF[r], aG[r]);
-          }
+          for (int r = 0; r < R; ++r) fwd_record<D>(q[r], p[r], v, aF[r], aG[r]);
         }
       }
 #pragma unroll
@@ -307,7 +494,8 @@ struct FwdTile {
 //   t = e~.d~ (= s e.d), m_j = alpha_j + t p_j, h = u + c t = alpha_i.p_j + p_i.m_j,
 //   A1 += g c e~,  A2 += g h d~,  B += g m_j;
 // dalpha = kq A1 - kappa A2 and dbeta = B.
-template <int R, int D = 3>
+// U: records loaded ahead of the ones in use (0: none).
+template <int R, int D = 3, int U = 0>
 struct BwdTile {
   float2 q[R][D], p[R][D], a[R][D], b[R][D];
   float s1[R][D], c1[R][D], s2[R][D], c2[R][D], sB[R][D], cB[R][D];
@@ -330,15 +518,19 @@ struct BwdTile {
 
   // Sources [lo, hi) of the staged chunk; lo is a multiple of 8.
   __device__ __forceinline__ void consume(const float4* const* bufs, int lo, int hi) {
+    if constexpr (U > 0)
+      consume_ahead(bufs, lo, hi);
+    else
+      consume_plain(bufs, lo, hi);
+  }
+
+  __device__ __forceinline__ void consume_plain(const float4* const* bufs, int lo, int hi) {
     const float4* Q = bufs[0];
     const float4* Ab = bufs[1];
     for (int sb = lo; sb < hi; sb += kSub) {
       const int sl = min(kSub, hi - sb);
       float2 a1[R][D], a2[R][D], bb[R][D];
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int k = 0; k < D; ++k) a1[r][k] = a2[r][k] = bb[r][k] = make_float2(0.f, 0.f);
+      zero(a1, a2, bb);
       for (int jj = 0; jj < sl; jj += kUnroll) {
 #pragma unroll
         for (int u = 0; u < kUnroll / 2; ++u) {
@@ -347,20 +539,68 @@ struct BwdTile {
           rec_split<D>(Q + ri, v);
           rec_split<D>(Ab + ri, w);
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            bwd_record<D>(q[r], p[r], a[r], b[r], v, w, a1[r], a2[r], bb[r]);
-          }
+          for (int r = 0; r < R; ++r) bwd_record<D>(q[r], p[r], a[r], b[r], v, w, a1[r], a2[r], bb[r]);
         }
       }
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          kahan_add(s1[r][k], c1[r][k], __fadd_rn(a1[r][k].x, a1[r][k].y));
-          kahan_add(s2[r][k], c2[r][k], __fadd_rn(a2[r][k].x, a2[r][k].y));
-          kahan_add(sB[r][k], cB[r][k], __fadd_rn(bb[r][k].x, bb[r][k].y));
-        }
+      fold(a1, a2, bb);
     }
+  }
+
+  // The same with the next U records on their way, across the sub-blocks.
+  __device__ __forceinline__ void consume_ahead(const float4* const* bufs, int lo, int hi) {
+    constexpr int V = U > 0 ? U : 1;
+    static_assert(kUnroll % (2 * V) == 0, "groups must divide the split granule");
+    const float4 *P = bufs[0] + lo / 2 * D, *PA = bufs[1] + lo / 2 * D;
+    float4 nx[V][D], ny[V][D];
+    load_records<V, D>(P, nx);
+    load_records<V, D>(PA, ny);
+    for (int sb = lo; sb < hi; sb += kSub) {
+      const int sl = min(kSub, hi - sb);
+      float2 a1[R][D], a2[R][D], bb[R][D];
+      zero(a1, a2, bb);
+      for (int jj = 0; jj < sl; jj += 2 * V) {
+        float4 cu[V][D], cy[V][D];
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+#pragma unroll
+          for (int f = 0; f < D; ++f) {
+            cu[u][f] = nx[u][f];
+            cy[u][f] = ny[u][f];
+          }
+        P += V * D;
+        PA += V * D;
+        load_records<V, D>(P, nx);
+        load_records<V, D>(PA, ny);
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+          float2 v[2 * D], w[2 * D];
+          rec_split<D>(cu[u], v);
+          rec_split<D>(cy[u], w);
+#pragma unroll
+          for (int r = 0; r < R; ++r) bwd_record<D>(q[r], p[r], a[r], b[r], v, w, a1[r], a2[r], bb[r]);
+        }
+      }
+      fold(a1, a2, bb);
+    }
+  }
+
+  __device__ __forceinline__ static void zero(float2 (&a1)[R][D], float2 (&a2)[R][D], float2 (&bb)[R][D]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int k = 0; k < D; ++k) a1[r][k] = a2[r][k] = bb[r][k] = make_float2(0.f, 0.f);
+  }
+
+  // Both halves of the plain sums into the Kahan pairs.
+  __device__ __forceinline__ void fold(const float2 (&a1)[R][D], const float2 (&a2)[R][D], const float2 (&bb)[R][D]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        kahan_add(s1[r][k], c1[r][k], __fadd_rn(a1[r][k].x, a1[r][k].y));
+        kahan_add(s2[r][k], c2[r][k], __fadd_rn(a2[r][k].x, a2[r][k].y));
+        kahan_add(sB[r][k], cB[r][k], __fadd_rn(bb[r][k].x, bb[r][k].y));
+      }
   }
 
   // out[0..D) = dalpha, out[D..2D) = dbeta of target r.

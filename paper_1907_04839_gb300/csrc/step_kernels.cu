@@ -194,7 +194,9 @@ __device__ __forceinline__ void push_tile(const float4 (&red)[W][M][D], float4* 
 // Accumulates this thread's H0 and mismatch contributions in hc, mc.
 // V: the variants (RK4 stages, the terminal launch) are compiled in.  D: the
 // dimension of the landmarks (3, or 2 for planar landmarks).
-template <int NT, int R, int W, bool V, int D>
+// Cull: ordered landmarks with the boxes of their runs; the CTA sums every
+// C-th run of sources, those out of its tile's reach left out.
+template <int NT, int R, int W, bool V, int D, bool Cull = false>
 __device__ __forceinline__ void forward_body(const StepFwdArgs& a, const StepView& v, double& hc, double& mc) {
   constexpr int TG = NT / W;  // threads per warp group
   constexpr int M = TG * R;   // targets of the CTA
@@ -226,6 +228,8 @@ __device__ __forceinline__ void forward_body(const StepFwdArgs& a, const StepVie
   const int j1 = min(j0 + v.split_len, lim);
   if (threadIdx.x == 0) pipe_init(pp, NT / 32);
   __syncthreads();
+  // Written before the sweep's first launch: readable before the wait.
+  const bool dense = Cull && *a.dense != 0;
   pdl_wait();  // the previous step's state must be complete
 
   const int tile0 = v.off + v.tile * M;
@@ -234,7 +238,18 @@ __device__ __forceinline__ void forward_body(const StepFwdArgs& a, const StepVie
   FwdTile<R, D> t;
   t.load(a.qp, tile0 + lt0, TG, lim);
   const float4* src[1] = {a.qp};
-  stream_sources<1, W, D>(sm.st, pp, src, j0, j1, t, a.status, grp);  // ends with a CTA barrier
+  if constexpr (Cull) {
+    __shared__ unsigned list[kListCap + 1];
+    const int nrun = v.npad / kGran;
+    sum_in_reach<1, D>(
+        sm.st, pp, src,
+        [&](int w0, int w1, unsigned* l) {
+          return list_for_tile<D, M>(a.box, tile0, nrun, static_cast<int>(rank), static_cast<int>(C), w0, w1, l);
+        },
+        nrun, static_cast<int>(rank), static_cast<int>(C), dense, j0, j1, t, list, a.status);
+  } else {
+    stream_sources<1, W, D>(sm.st, pp, src, j0, j1, t, a.status, grp);  // ends with a CTA barrier
+  }
   const int slice = (M + static_cast<int>(C) - 1) / static_cast<int>(C);  // the last CTA may reduce fewer
   const auto res = [&](const FwdTile<R, D>& tt, int r, ds* w) { tt.result(r, v.kappa_f, w); };
   combine_tile<NT, R, W, M, D>(sm.red, t, res, lt0, grp);
@@ -322,8 +337,10 @@ __device__ __forceinline__ void forward_body(const StepFwdArgs& a, const StepVie
     }
     if (!isfinite(q) || !isfinite(p)) atomicOr(a.status, kErrNonFinite);
     float* qn = reinterpret_cast<float*>(a.qp_next + (i >> 1) * D) + 2 * k + (i & 1);
-    qn[0] = -(float)(v.kq * q);
+    const float vq = -(float)(v.kq * q);
+    qn[0] = vq;
     qn[2 * D] = (float)p;
+    if (Cull && a.box_next && !dense) box_add(a.box_next, i, k, vq);
     if (a.last && a.with_loss) {
       const double r = q - a.t64[tt];
       mc += r * r;
@@ -345,7 +362,8 @@ __device__ __forceinline__ void forward_body(const StepFwdArgs& a, const StepVie
 // requires C | M; compiled that way the whole kernel ran 2% faster on GB300
 // (N = 4096 and 16384, same cluster shape), so clusters that divide the tile
 // use it and the others a separate instantiation.
-template <int NT, int R, int W, bool V, int D, bool Ragged = false>
+// Waves: the grid has several waves (the pair loop loads ahead).
+template <int NT, int R, int W, bool V, int D, bool Ragged = false, bool Cull = false, bool Waves = Cull>
 __device__ __forceinline__ void backward_body(const StepBwdArgs& a, const StepView& v) {
   constexpr int TG = NT / W;  // threads per warp group
   constexpr int M = TG * R;   // targets of the CTA
@@ -382,18 +400,31 @@ __device__ __forceinline__ void backward_body(const StepBwdArgs& a, const StepVi
   const int j1 = min(j0 + v.split_len, lim);
   if (threadIdx.x == 0) pipe_init(pp, NT / 32);
   __syncthreads();
+  const bool dense = Cull && *a.dense != 0;
   pdl_wait();
 
   const int tile0 = v.off + v.tile * M;
   const int grp = W == 1 ? 0 : static_cast<int>(threadIdx.x) / TG;
   const int lt0 = W == 1 ? static_cast<int>(threadIdx.x) : static_cast<int>(threadIdx.x) % TG;
-  BwdTile<R, D> t;
+  using BTile = BwdTile<R, D, Waves && NT == 64 && R == 1 && W == 1 ? kAhead : 0>;
+  BTile t;
   t.load(a.qp, a.ab, tile0 + lt0, TG, lim);
   const float4* src[2] = {a.qp, a.ab};
-  stream_sources<2, W, D>(sm.st, pp, src, j0, j1, t, a.status, grp);
+  if constexpr (Cull) {
+    __shared__ unsigned list[kListCap + 1];
+    const int nrun = v.npad / kGran;
+    sum_in_reach<2, D>(
+        sm.st, pp, src,
+        [&](int w0, int w1, unsigned* l) {
+          return list_for_tile<D, M>(a.box, tile0, nrun, static_cast<int>(rank), static_cast<int>(C), w0, w1, l);
+        },
+        nrun, static_cast<int>(rank), static_cast<int>(C), dense, j0, j1, t, list, a.status);
+  } else {
+    stream_sources<2, W, D>(sm.st, pp, src, j0, j1, t, a.status, grp);
+  }
   const int slice = Ragged ? (M + static_cast<int>(C) - 1) / static_cast<int>(C) : M / static_cast<int>(C);
   if constexpr (kPush) {
-    const auto res = [&](const BwdTile<R, D>& tt, int r, ds* w) { tt.result(r, v.kq_f, v.kappa_f, w); };
+    const auto res = [&](const BTile& tt, int r, ds* w) { tt.result(r, v.kq_f, v.kappa_f, w); };
     combine_tile<NT, R, W, M, D>(sm.red, t, res, lt0, grp);
     cluster_wait();  // every peer's receive buffer exists
     push_tile<NT, R, W, M, D>(sm.red, recv, t, res, lt0, rank, slice);
@@ -486,9 +517,10 @@ __device__ __forceinline__ void backward_body(const StepBwdArgs& a, const StepVi
     }
     if (a.first) {
       const double gp = be + (a.h_at_end ? 0.0 : a.hp0[tt]);
-      if (a.grad_p0) a.grad_p0[tt] = (float)gp;
-      if (a.grad_p0_64) a.grad_p0_64[tt] = gp;
-      if (a.grad_q0) a.grad_q0[tt] = (float)(al + (a.h_at_end ? 0.0 : a.hq0[tt]));
+      const int to = Cull ? D * a.perm[i] + k : tt;  // in the caller's order
+      if (a.grad_p0) a.grad_p0[to] = (float)gp;
+      if (a.grad_p0_64) a.grad_p0_64[to] = gp;
+      if (a.grad_q0) a.grad_q0[to] = (float)(al + (a.h_at_end ? 0.0 : a.hq0[tt]));
     }
   }
   if constexpr (!kPush) cluster_sync();  // peers may still be reading this CTA's partials
@@ -499,8 +531,8 @@ __device__ __forceinline__ void backward_body(const StepBwdArgs& a, const StepVi
 // kinetic term at t = 0), true with the variants compiled in (RK4 stages, the
 // terminal launch).  Keeping them apart leaves the plain kernels' register
 // allocation as the pair loop needs it.
-template <int NT, int R, int W, bool V, int D = 3>
-__global__ void __launch_bounds__(NT) k_step_forward(StepFwdArgs a) {
+template <int NT, int R, int W, bool V, int D = 3, bool Cull = false>
+__global__ void __launch_bounds__(NT, Cull && NT == 128 && !V ? 8 : 0) k_step_forward(StepFwdArgs a) {
   __shared__ double shred[NT / 32];
   __shared__ int am_last;
   StepView v;
@@ -516,7 +548,7 @@ __global__ void __launch_bounds__(NT) k_step_forward(StepFwdArgs a) {
   v.dt = a.dt;
   v.lambda = a.lambda;
   double hc = 0.0, mc = 0.0;
-  forward_body<NT, R, W, V, D>(a, v, hc, mc);
+  forward_body<NT, R, W, V, D, Cull>(a, v, hc, mc);
   const bool reduce_h = a.first || a.terminal;
   const bool reduce_m = a.last && a.with_loss;
   if ((!reduce_h && !reduce_m) || a.dry) return;  // uniform across the grid
@@ -533,7 +565,7 @@ __global__ void __launch_bounds__(NT) k_step_forward(StepFwdArgs a) {
   }
 }
 
-template <int NT, int R, int W, bool V, int D = 3, bool Ragged = false>
+template <int NT, int R, int W, bool V, int D = 3, bool Ragged = false, bool Cull = false>
 __global__ void __launch_bounds__(NT) k_step_backward(StepBwdArgs a) {
   StepView v;
   v.off = 0;
@@ -547,7 +579,7 @@ __global__ void __launch_bounds__(NT) k_step_backward(StepBwdArgs a) {
   v.kappa = a.kappa64;
   v.dt = a.dt;
   v.lambda = 0.0;
-  backward_body<NT, R, W, V, D, Ragged>(a, v);
+  backward_body<NT, R, W, V, D, Ragged, Cull>(a, v);
 }
 
 // ---------------------------------------------------------------- packed batch kernels
@@ -592,7 +624,7 @@ __global__ void __launch_bounds__(NT) k_bstep_forward(StepFwdArgs a, BatchTables
 
 template <int NT, int R, int W>
 __global__ void __launch_bounds__(NT) k_bstep_backward(StepBwdArgs a, BatchTables bt) {
-  backward_body<NT, R, W, false, 3>(a, batch_view(bt, true));
+  backward_body<NT, R, W, false, 3, false, false, true>(a, batch_view(bt, true));
 }
 
 // ---------------------------------------------------------------- host side
@@ -739,7 +771,9 @@ bool late_trigger_for(int kind, const StepConfig& c, int dim, bool rk) {
   // (+13% forward-sweep time at N = 4096 with the trigger).  Residency is
   // that of the instantiation the launch runs (the uneven-cluster, RK4 and
   // planar kernels differ in registers and shared memory).
-  if (kind != 1) return false;
+  // Culling reverse steps neither: 31.5 us without, 35.6 with it, at
+  // N = 4096.
+  if (kind != 1 || c.cull) return false;
   const BwdKernel kern = backward_kernel_for(c, dim, rk);
   if (!kern) return false;
   int dev = 0;
@@ -936,7 +970,37 @@ cudaError_t launch_bstep_backward(const StepConfig& c, int items, const StepBwdA
 // (RK4 stages, the terminal launch) go to the V = true instantiation of the
 // built-in configuration's kernel variant; planar landmarks (dim 2) to the
 // D = 2 instantiations of that variant.  Null: no instantiation exists.
+namespace {
+// The culling instantiations: the CTA sizes of the built-in configurations.
+FwdKernel cull_forward_kernel(const StepConfig& c, int dim, bool variants) {
+  if (c.R != 1 || c.groups != 1) return nullptr;
+  if (c.threads == kVarFwdThreads) {
+    if (dim == 2)
+      return variants ? k_step_forward<kVarFwdThreads, 1, 1, true, 2, true>
+                      : k_step_forward<kVarFwdThreads, 1, 1, false, 2, true>;
+    return variants ? k_step_forward<kVarFwdThreads, 1, 1, true, 3, true>
+                    : k_step_forward<kVarFwdThreads, 1, 1, false, 3, true>;
+  }
+  if (c.threads == kVarFwdThreads / 2 && dim == 3 && !variants) return k_step_forward<kVarFwdThreads / 2, 1, 1, false, 3, true>;
+  return nullptr;
+}
+
+template <bool Ragged>
+BwdKernel cull_backward_kernel(const StepConfig& c, int dim, bool rk) {
+  if (c.threads == kVarBwdThreads) {
+    if (dim == 2)
+      return rk ? k_step_backward<kVarBwdThreads, 1, 1, true, 2, Ragged, true>
+                : k_step_backward<kVarBwdThreads, 1, 1, false, 2, Ragged, true>;
+    return rk ? k_step_backward<kVarBwdThreads, 1, 1, true, 3, Ragged, true>
+              : k_step_backward<kVarBwdThreads, 1, 1, false, 3, Ragged, true>;
+  }
+  if (c.threads == kVarBwdThreads / 2 && dim == 3 && !rk) return k_step_backward<kVarBwdThreads / 2, 1, 1, false, 3, Ragged, true>;
+  return nullptr;
+}
+}  // namespace
+
 FwdKernel forward_kernel_for(const StepConfig& c, int dim, bool variants) {
+  if (c.cull) return cull_forward_kernel(c, dim, variants);
   if (dim == 2) {  // planar landmarks: the built-in configuration only
     if (c.threads != kVarFwdThreads || c.R != 1 || c.groups != 1) return nullptr;
     return variants ? k_step_forward<kVarFwdThreads, 1, 1, true, 2> : k_step_forward<kVarFwdThreads, 1, 1, false, 2>;
@@ -953,6 +1017,10 @@ FwdKernel forward_kernel_for(const StepConfig& c, int dim, bool variants) {
 }
 
 BwdKernel backward_kernel_for(const StepConfig& c, int dim, bool rk) {
+  if (c.cull) {
+    if (c.R != 1 || c.groups != 1) return nullptr;
+    return c.threads % c.cluster ? cull_backward_kernel<true>(c, dim, rk) : cull_backward_kernel<false>(c, dim, rk);
+  }
   if ((c.threads / c.groups * c.R) % c.cluster != 0) {  // the instantiations for clusters that do not divide the tile
     if (c.R != 1 || c.groups != 1 || (c.threads != 32 && c.threads != kVarBwdThreads)) return nullptr;
     if (dim == 2) {
