@@ -93,11 +93,16 @@ struct VelArgs {
   float* v_out;      // velocity out (m x 3), or null for an Euler step
   int m, npad, split_len;
   double kq, dt;
+  const unsigned* box;  // boxes of the landmarks' runs (Cull)
   unsigned* status;
 };
 
 constexpr int kVM = kVT * kVR;  // query points per CTA
 
+// Cull: landmarks in spatial order; runs of them out of the reach of the
+// tile's points are left out.  Points that are neighbours in the caller's
+// array (a grid, a mesh) have small boxes; scattered ones cost the test alone.
+template <bool Cull>
 __global__ void __launch_bounds__(kVT) k_velocity(VelArgs a) {
   union Smem {
     StageBuf<1> st;
@@ -123,7 +128,50 @@ __global__ void __launch_bounds__(kVT) k_velocity(VelArgs a) {
   VelTile<kVR> t;
   t.load(a.x64, tile0 + static_cast<int>(threadIdx.x), kVT, a.m, a.kq);
   const float4* src[1] = {a.qp};
-  stream_sources<1>(sm.st, pp, src, j0, j1, t, a.status);  // ends with a CTA barrier
+  if constexpr (Cull) {
+    __shared__ unsigned list[kListCap + 1];
+    __shared__ float wbox[kVT / 32][6];
+    // Box of the tile's points, as record positions (negated).
+    RunBox<3> tb;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      tb.hi[k] = tb.lo[k] = -INFINITY;
+#pragma unroll
+      for (int r = 0; r < kVR; ++r) {
+        if (tile0 + static_cast<int>(threadIdx.x) + r * kVT < a.m) {
+          const float q = t.q[r][k].x;
+          const bool nan = q != q;  // everything stays in reach: the NaN must show
+          tb.hi[k] = fmaxf(tb.hi[k], nan ? INFINITY : -q);
+          tb.lo[k] = fmaxf(tb.lo[k], nan ? INFINITY : q);
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        tb.hi[k] = fmaxf(tb.hi[k], __shfl_xor_sync(0xffffffffu, tb.hi[k], o));
+        tb.lo[k] = fmaxf(tb.lo[k], __shfl_xor_sync(0xffffffffu, tb.lo[k], o));
+      }
+      if ((threadIdx.x & 31) == 0) {
+        wbox[threadIdx.x >> 5][k] = tb.hi[k];
+        wbox[threadIdx.x >> 5][3 + k] = tb.lo[k];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int w = 0; w < kVT / 32; ++w) {
+        tb.hi[k] = fmaxf(tb.hi[k], wbox[w][k]);
+        tb.lo[k] = fmaxf(tb.lo[k], wbox[w][3 + k]);
+      }
+    sum_in_reach<1, 3>(
+        sm.st, pp, src,
+        [&](int w0, int w1, unsigned* l) {
+          return list_for_box<3>(a.box, tb, static_cast<int>(rank), static_cast<int>(C), w0, w1, l);
+        },
+        a.npad / kGran, static_cast<int>(rank), static_cast<int>(C), false, j0, j1, t, list, a.status);
+  } else {
+    stream_sources<1>(sm.st, pp, src, j0, j1, t, a.status);  // ends with a CTA barrier
+  }
 #pragma unroll
   for (int r = 0; r < kVR; ++r) {
     const ds f0 = ds_from_kahan(t.sF[r][0], t.cF[r][0]);
@@ -203,7 +251,9 @@ cudaError_t launch_velocity(const VelConfig& c, const VelArgs& a, cudaStream_t s
   {
     std::lock_guard<std::mutex> lk(g_vel_attr_mu);
     if (!g_vel_attr_done) {
-      const cudaError_t e = cudaFuncSetAttribute(k_velocity, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      cudaError_t e = cudaFuncSetAttribute(k_velocity<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_velocity<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e != cudaSuccess) return e;
       g_vel_attr_done = true;
     }
@@ -230,7 +280,7 @@ cudaError_t launch_velocity(const VelConfig& c, const VelArgs& a, cudaStream_t s
   }
   cfg.attrs = at;
   cfg.numAttrs = k;
-  return cudaLaunchKernelEx(&cfg, k_velocity, a);
+  return a.box ? cudaLaunchKernelEx(&cfg, k_velocity<true>, a) : cudaLaunchKernelEx(&cfg, k_velocity<false>, a);
 }
 
 // Room for m points (FP64 state and FP32 staging in and out).
@@ -286,13 +336,32 @@ extern "C" gs_status velocity_field(int64_t N, int64_t M, double sigma, const fl
   if ((s = stage_in(p, w->in_p, n3, st, &dp, &host)) != GS_OK) return s;
   if ((s = stage_in(x, w->pts_in, m3, st, &dx, &host)) != GS_OK) return s;
   const KernelScales sc = make_scales(sigma);
-  const RecordSet qp{dq, dp, w->traj, sc.kq, 1.0, 0};
-  GS_CUDA(launch_to_records(&qp, 1, n, npad, w->status, st));
+  // Enough pairs to pay for the order of the landmarks (one launch more and N
+  // codes read per landmark): 10^9 are 350 us of pair sums.
+  const bool ordered = npad >= 1024 && m >= n && static_cast<double>(n) * m >= 1e9;
+  if (ordered) {
+    if ((s = reserve_order(*w, npad, box_words(npad))) != GS_OK) return s;
+    PackArgs pk{};
+    pk.q = dq;
+    pk.p = dp;
+    pk.q64 = w->q64;
+    pk.p64 = w->p64;
+    pk.qp = w->traj;
+    pk.n = n;
+    pk.kq = sc.kq;
+    pk.status = w->status;
+    pk.npad = npad;
+    GS_CUDA(launch_order_pack(pk, w->codes, w->perm, w->boxes, box_words(npad), w->dense, st));
+  } else {
+    const RecordSet qp{dq, dp, w->traj, sc.kq, 1.0, 0};
+    GS_CUDA(launch_to_records(&qp, 1, n, npad, w->status, st));
+  }
   w->clean_n = -1;  // record slot 0 was overwritten
   k_points_to64<<<conv_blocks(m3), 256, 0, st>>>(dx, w->pts64, m3);
   GS_CUDA(cudaGetLastError());
   const VelConfig c = vel_config(m, npad, w->num_sms);
-  VelArgs a{w->traj, w->pts64, w->pts_out, m, npad, c.split_len, sc.kq, 0.0, w->status};
+  VelArgs a{w->traj, w->pts64, w->pts_out, m, npad, c.split_len, sc.kq, 0.0,
+            ordered ? w->boxes : nullptr, w->status};
   GS_CUDA(launch_velocity(c, a, st, false));
   bool want_sync = host;
   if ((s = copy_out(v, w->pts_out, m3, st, &want_sync)) != GS_OK) return s;
@@ -332,9 +401,11 @@ extern "C" gs_status flow_points(const gs_params* prm, const float* q0, const fl
   k_points_to64<<<conv_blocks(m3), 256, 0, st>>>(dx, w->pts64, m3);
   GS_CUDA(cudaGetLastError());
   const VelConfig c = vel_config(m, npad, w->num_sms);
+  // The test of the runs takes about 1 us a CTA: worth it from 1024 landmarks a CTA.
+  const bool ordered = c.split_len >= 1024 && !small_path(*w, *prm) && use_order(npad, T, 3);
   for (int k = 0; k < T; ++k) {
     VelArgs a{w->traj + static_cast<size_t>(k) * w->slot(), w->pts64, nullptr, m, npad, c.split_len, sc.kq,
-              1.0 / T, w->status};
+              1.0 / T, ordered ? w->boxes + k * box_words(npad) : nullptr, w->status};
     GS_CUDA(launch_velocity(c, a, st, k > 0));
   }
   k_points_to32<<<conv_blocks(m3), 256, 0, st>>>(w->pts64, w->pts_out, m3);
