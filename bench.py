@@ -58,7 +58,7 @@ FLOPS_PER_PAIR_FWD = 27
 FLOPS_PER_PAIR_BWD = 63
 # FP32 instructions per pair issued by the kernels (for the pipe fraction).
 INSTR_PER_PAIR_FWD = 16
-INSTR_PER_PAIR_BWD = 36
+INSTR_PER_PAIR_BWD = 35
 # The velocity field of Eq. 4 per (point, landmark) pair: difference (3),
 # squared distance (5), exponent scale (1), g p_j accumulated (6); issued
 # FP32 lane-operations 9.
@@ -666,12 +666,14 @@ def _timed_gradients(lib, prm, bufs, stream, reps, flush):
     return float(np.median(tt)), float(np.median(fw)), float(np.median(bw))
 
 
-def roofline_at(gsh, lib, dev, n, peak, mufu_peak, T=T_STEPS, sigma=0.05, reps=8):
+def roofline_at(gsh, lib, dev, n, peak, mufu_peak, T=T_STEPS, sigma=0.2, reps=8):
     """The step kernels' roofline at a larger N (16384 landmarks: several
     waves per launch, where the pair loops rather than the fixed per-launch
     costs set the time): whole gradients of an ellipsoid workload
-    (sigma = 0.05, T = 20), per-launch times from the graph's phase events
-    (sweep / T)."""
+    (T = 20), per-launch times from the graph's phase events (sweep / T).
+    sigma = 0.2 has nearly every pair in reach, so every pair is evaluated
+    and the counts are of work done; at narrower kernels this size leaves out
+    pairs whose Gaussian is exactly zero."""
     import torch
     q, p, t = _grad_inputs(dev, n)
     bufs = (q, p, t, torch.empty_like(q), torch.empty_like(q))
