@@ -8,9 +8,10 @@
 //  * the reduction scratch and the device status word;
 //  * a cache of instantiated CUDA graphs.
 // Each graph holds the T forward steps, and for gradients also the T reverse
-// steps: a pair-sum kernel followed by a combine kernel per step, linked by
-// programmatic dependent launch.  A call packs the inputs, replays the
-// graph, then copies the outputs out.
+// steps: one fused kernel per step, linked by programmatic dependent launch.
+// A call packs the inputs (large ones in spatial order, order.cu), replays the
+// graph, then copies the outputs out.  Small problems run as one launch
+// without a graph (small.cu).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -603,9 +604,7 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
   return GS_OK;
 }
 
-// Where a call's kernels write a caller's output: the array itself when it is
-// this device's memory, else the staging buffer (copied out afterwards).
-static gs_status out_ptr(float* user, float* staging, float** dev) {
+gs_status out_ptr(float* user, float* staging, float** dev) {
   *dev = nullptr;
   if (!user) return GS_OK;
   const PtrKind kind = pointer_kind(user);

@@ -156,6 +156,9 @@ gs_status ensure_clean(Workspace& w, int n, cudaStream_t st, int dim = 3);
 bool is_device_ptr(const void* p);
 gs_status stage_in(const float* src, float* staging, size_t n3, cudaStream_t st, const float** dev, bool* host);
 gs_status copy_out(float* dst, const float* src, size_t n3, cudaStream_t st, bool* host);
+// Where a call's kernels write a caller's output: the array itself when it is
+// this device's memory, else the staging buffer (copied out afterwards).
+gs_status out_ptr(float* user, float* staging, float** dev);
 // Wait for the stream; the scalars are in w.host afterwards, the status word
 // is read and cleared.
 gs_status finish_sync(Workspace& w, cudaStream_t st);

@@ -88,7 +88,6 @@ PairConfig choose_forward_config(int npad, int num_sms);
 // picks the balanced split count.  threads == 0 in the result: no such variant.
 PairConfig forward_config_for(int npad, int num_sms, int threads, int R, int splits);
 PairConfig backward_config_for(int npad, int num_sms, int threads, int R, int splits);
-PairConfig choose_backward_config(int npad, int num_sms);
 // Forward configuration with at most `max_splits` source splits.
 PairConfig choose_forward_config_capped(int npad, int num_sms, int max_splits);
 

@@ -36,13 +36,15 @@ struct VelTile {
   float2 q[R][3];  // prescaled points, duplicated for the paired lanes
   float sF[R][3], cF[R][3];
 
-  __device__ __forceinline__ void load(const double* x64, int base, int stride, int m, double kq) {
+  // Points from the FP64 state x64, or where that is null from the caller's x32.
+  __device__ __forceinline__ void load(const double* x64, const float* x32, int base, int stride, int m, double kq) {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int i = base + r * stride;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const float v = i < m ? static_cast<float>(kq * x64[3 * static_cast<size_t>(i) + k]) : 0.f;
+        const size_t t = 3 * static_cast<size_t>(i) + k;
+        const float v = i < m ? static_cast<float>(kq * (x64 ? x64[t] : static_cast<double>(x32[t]))) : 0.f;
         q[r][k] = dup(v);
         sF[r][k] = cF[r][k] = 0.f;
       }
@@ -89,8 +91,9 @@ struct VelTile {
 
 struct VelArgs {
   const float4* qp;  // QP pair records of the landmark state (npad landmarks)
-  double* x64;       // points, FP64 (m x 3); moved in place when v_out is null
-  float* v_out;      // velocity out (m x 3), or null for an Euler step
+  double* x64;       // points, FP64 (m x 3), moved in place; null: read x32, write v_out
+  const float* x32;
+  float* v_out;      // velocity out (m x 3); null for an Euler step
   int m, npad, split_len;
   double kq, dt;
   const unsigned* box;  // boxes of the landmarks' runs (Cull)
@@ -126,7 +129,7 @@ __global__ void __launch_bounds__(kVT) k_velocity(VelArgs a) {
 
   const int tile0 = blockIdx.y * kVM;
   VelTile<kVR> t;
-  t.load(a.x64, tile0 + static_cast<int>(threadIdx.x), kVT, a.m, a.kq);
+  t.load(a.x64, a.x32, tile0 + static_cast<int>(threadIdx.x), kVT, a.m, a.kq);
   const float4* src[1] = {a.qp};
   if constexpr (Cull) {
     __shared__ unsigned list[kListCap + 1];
@@ -163,12 +166,24 @@ __global__ void __launch_bounds__(kVT) k_velocity(VelArgs a) {
         tb.hi[k] = fmaxf(tb.hi[k], wbox[w][k]);
         tb.lo[k] = fmaxf(tb.lo[k], wbox[w][3 + k]);
       }
+    // A tile of scattered points reaches everything: 32 runs spread over the
+    // landmarks tell, and the plain stream costs less than testing every run
+    // and copying them one by one (7 to 15 % at 12000 to 40000 landmarks).
+    const int nrun = a.npad / kGran;
+    if (threadIdx.x < 32) {
+      const int run = static_cast<int>(static_cast<long long>(threadIdx.x) * nrun / 32);
+      const bool all = __all_sync(0xffffffffu, in_reach(tb, run_box<3>(load_box(a.box, run))));
+      if (threadIdx.x == 0) list[kListCap] = all;
+    }
+    __syncthreads();
+    const bool dense = list[kListCap] != 0;
+    __syncthreads();
     sum_in_reach<1, 3>(
         sm.st, pp, src,
         [&](int w0, int w1, unsigned* l) {
           return list_for_box<3>(a.box, tb, static_cast<int>(rank), static_cast<int>(C), w0, w1, l);
         },
-        a.npad / kGran, static_cast<int>(rank), static_cast<int>(C), false, j0, j1, t, list, a.status);
+        nrun, static_cast<int>(rank), static_cast<int>(C), dense, j0, j1, t, list, a.status);
   } else {
     stream_sources<1>(sm.st, pp, src, j0, j1, t, a.status);  // ends with a CTA barrier
   }
@@ -335,10 +350,13 @@ extern "C" gs_status velocity_field(int64_t N, int64_t M, double sigma, const fl
   if ((s = stage_in(q, w->in_q, n3, st, &dq, &host)) != GS_OK) return s;
   if ((s = stage_in(p, w->in_p, n3, st, &dp, &host)) != GS_OK) return s;
   if ((s = stage_in(x, w->pts_in, m3, st, &dx, &host)) != GS_OK) return s;
+  float* dv = nullptr;
+  if ((s = out_ptr(v, w->pts_out, &dv)) != GS_OK) return s;
   const KernelScales sc = make_scales(sigma);
-  // Enough pairs to pay for the order of the landmarks (one launch more and N
-  // codes read per landmark): 10^9 are 350 us of pair sums.
-  const bool ordered = npad >= 1024 && m >= n && static_cast<double>(n) * m >= 1e9;
+  // The order of the landmarks reads N codes per landmark and takes one launch
+  // more: under 2 % of the pair sums from 64 points a landmark and 10^9 pairs
+  // (350 us) on.
+  const bool ordered = npad >= 1024 && m / 64 >= n && static_cast<double>(n) * m >= 1e9;
   if (ordered) {
     if ((s = reserve_order(*w, npad, box_words(npad))) != GS_OK) return s;
     PackArgs pk{};
@@ -357,14 +375,12 @@ extern "C" gs_status velocity_field(int64_t N, int64_t M, double sigma, const fl
     GS_CUDA(launch_to_records(&qp, 1, n, npad, w->status, st));
   }
   w->clean_n = -1;  // record slot 0 was overwritten
-  k_points_to64<<<conv_blocks(m3), 256, 0, st>>>(dx, w->pts64, m3);
-  GS_CUDA(cudaGetLastError());
+  // The points are read and the velocities written where the caller keeps them.
   const VelConfig c = vel_config(m, npad, w->num_sms);
-  VelArgs a{w->traj, w->pts64, w->pts_out, m, npad, c.split_len, sc.kq, 0.0,
-            ordered ? w->boxes : nullptr, w->status};
-  GS_CUDA(launch_velocity(c, a, st, false));
+  VelArgs a{w->traj, nullptr, dx, dv, m, npad, c.split_len, sc.kq, 0.0, ordered ? w->boxes : nullptr, w->status};
+  GS_CUDA(launch_velocity(c, a, st, true));
   bool want_sync = host;
-  if ((s = copy_out(v, w->pts_out, m3, st, &want_sync)) != GS_OK) return s;
+  if (dv != v && (s = copy_out(v, dv, m3, st, &want_sync)) != GS_OK) return s;
   if (want_sync) return finish_sync(*w, st);
   return GS_OK;
 }
@@ -404,14 +420,16 @@ extern "C" gs_status flow_points(const gs_params* prm, const float* q0, const fl
   // The test of the runs takes about 1 us a CTA: worth it from 1024 landmarks a CTA.
   const bool ordered = c.split_len >= 1024 && !small_path(*w, *prm) && use_order(npad, T, 3);
   for (int k = 0; k < T; ++k) {
-    VelArgs a{w->traj + static_cast<size_t>(k) * w->slot(), w->pts64, nullptr, m, npad, c.split_len, sc.kq,
+    VelArgs a{w->traj + static_cast<size_t>(k) * w->slot(), w->pts64, nullptr, nullptr, m, npad, c.split_len, sc.kq,
               1.0 / T, ordered ? w->boxes + k * box_words(npad) : nullptr, w->status};
     GS_CUDA(launch_velocity(c, a, st, k > 0));
   }
-  k_points_to32<<<conv_blocks(m3), 256, 0, st>>>(w->pts64, w->pts_out, m3);
+  float* dx1 = nullptr;
+  if ((s = out_ptr(x1, w->pts_out, &dx1)) != GS_OK) return s;
+  k_points_to32<<<conv_blocks(m3), 256, 0, st>>>(w->pts64, dx1, m3);
   GS_CUDA(cudaGetLastError());
   bool want_sync = host;
-  if ((s = copy_out(x1, w->pts_out, m3, st, &want_sync)) != GS_OK) return s;
+  if (dx1 != x1 && (s = copy_out(x1, dx1, m3, st, &want_sync)) != GS_OK) return s;
   if (want_sync) return finish_sync(*w, st);
   return GS_OK;
 }

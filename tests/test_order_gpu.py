@@ -82,3 +82,28 @@ def test_ordered_flow_comes_back_in_the_callers_order(n, dim):
     a, b = run(), every_pair(run)
     bar = BAR + 2.0 ** -24 * float(q.abs().max()) * 0.85 / 0.05
     assert rel(a[0], b[0]) < bar and rel(a[1], b[1]) < bar and abs(a[2] - b[2]) < BAR * abs(b[2])
+
+
+@pytest.mark.parametrize("points", ["grid", "scattered"])
+def test_large_velocity_field_equals_its_slices(points):
+    """A field of many points orders its landmarks and leaves runs out of reach
+    out; fields of its slices (under 64 points a landmark) do not."""
+    n, sigma = 4097, 0.05
+    q, p, _ = case(n, "surface", 3)
+    if points == "grid":
+        g = torch.linspace(-1.2, 1.2, 65, device="cuda")
+        x = torch.stack(torch.meshgrid(g, g, g, indexing="ij"), dim=-1).reshape(-1, 3).contiguous()
+    else:
+        x = torch.rand((262300, 3), device="cuda", generator=torch.Generator("cuda").manual_seed(5)) * 2 - 1
+    v = gs().velocity_field(q, p, x, sigma)
+    parts = torch.cat([gs().velocity_field(q, p, c.contiguous(), sigma) for c in x.split(60001)])
+    assert rel(v, parts) < BAR
+
+
+def test_large_velocity_field_reports_a_nan_point():
+    q, p, _ = case(4097, "surface", 3)
+    x = np.random.default_rng(0).uniform(-1, 1, size=(262300, 3)).astype(np.float32)
+    x[100000, 2] = np.nan
+    with pytest.raises(gs().GShootError) as e:
+        gs().velocity_field(q.cpu().numpy(), p.cpu().numpy(), x, 0.05)
+    assert e.value.status == -5
