@@ -482,10 +482,11 @@ int shoot_ckpt(const Workspace& w, const gs_params& prm) {
 // against 47.9, 47.0, 47.1; 5000 64.0 against 51.9, 64.9, 64.9; 16384 489 against
 // 233, 477, 493; planar (0.05, 0.1) N = 3000 28.2 against 23.8, 30.0; 4096 38.6
 // against 30.1, 38.1.  The order itself takes about 10 us a call: a sweep has 10^9
-// pairs (1 ms) at least.  The rule must not depend on what a sweep computes:
+// pairs (1 ms) at least, and 8 evaluations, as ranking the landmarks reads N^2
+// codes.  The rule must not depend on what a sweep computes:
 // register compares the positions of a flow with a gradient's targets.
 bool use_order(int npad, int J, int dim) {
-  return npad >= (dim == 2 ? kOrderNpad2 : kOrderNpad) && static_cast<double>(J) * npad * npad >= 1e9 && (J + 1) * box_words(npad) * sizeof(unsigned) <= (size_t{1} << 30) && !step_override_set();
+  return npad >= (dim == 2 ? kOrderNpad2 : kOrderNpad) && J >= 8 && static_cast<double>(J) * npad * npad >= 1e9 && (J + 1) * box_words(npad) * sizeof(unsigned) <= (size_t{1} << 30) && !step_override_set();
 }
 
 gs_status reserve_order(Workspace& w, int npad, size_t nbox) {

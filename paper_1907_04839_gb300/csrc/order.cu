@@ -11,7 +11,7 @@
 // "Programming the Hilbert curve", 2004), in cells of a quarter of the
 // prescaled unit around landmark 0.  k_rank_pack: each landmark's rank in
 // (code, index) order by counting, then the pack of the caller's arrays at
-// that rank.  Counting reads N codes per landmark, two integer instructions
+// that rank.  Counting reads N codes per landmark, about three integer instructions
 // a pair against 51 for one time step's sums, needs no scratch and
 // no further launch, and gives the same order on every run.
 #include <algorithm>
@@ -23,7 +23,7 @@ namespace gs {
 namespace {
 
 constexpr int kOT = 256;
-constexpr int kLanes = 8;  // lanes that count for one landmark
+constexpr int kLanes = 8;  // lanes that count for two landmarks
 constexpr int kTile4 = 8 * kOT;  // uint4 of codes staged at a time (32 KB)
 
 template <int D>
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kOT) k_codes(const float* q, int n, float kq, 
   const int np = (n + 31) & ~31;
   for (size_t i = t0; i < static_cast<size_t>(np); i += static_cast<size_t>(gridDim.x) * kOT) {
     if (i >= static_cast<size_t>(n)) {
-      codes[i] = 0xffffffffu;
+      codes[i] = 0x7fffffffu;
       continue;
     }
     constexpr int B = 30 / D;
@@ -112,15 +112,16 @@ __device__ __forceinline__ bool mostly_in_reach(const unsigned* boxes, int npad)
 
 template <int D>
 __device__ __forceinline__ void rank_pack(const PackArgs& a, const unsigned* codes, int* perm, unsigned* boxes) {
+  // Eight lanes count for landmarks 2 g and 2 g + 1, each over every eighth
+  // group of four codes.
   const int gt = blockIdx.x * kOT + threadIdx.x;
-  const int i = gt / kLanes, lane = gt % kLanes;
-  const bool valid = i < a.n;
-  unsigned rank = 0;
+  const int i0 = 2 * (gt / kLanes), lane = gt % kLanes;
   // Codes pass through shared memory, a tile at a time: from L2 directly, few
   // loads in flight made this 15 us at N = 4096.
-  __shared__ uint4 tile[kTile4];
-  const unsigned ci = valid ? codes[i] : 0u;
-  const uint4* c4 = reinterpret_cast<const uint4*>(codes);
+  __shared__ int4 tile[kTile4];
+  const int c0 = i0 < a.n ? static_cast<int>(codes[i0]) : 0, c1 = i0 + 1 < a.n ? static_cast<int>(codes[i0 + 1]) : 0;
+  int n0 = 0, n1 = 0;
+  const int4* c4 = reinterpret_cast<const int4*>(codes);
   const int n4 = ((a.n + 31) & ~31) / 4;
   for (int t0 = 0; t0 < n4; t0 += kTile4) {
     const int len = min(kTile4, n4 - t0);
@@ -129,24 +130,40 @@ __device__ __forceinline__ void rank_pack(const PackArgs& a, const unsigned* cod
     for (int u = 0; u < kTile4 / kOT; ++u)
       if (threadIdx.x + u * kOT < len) tile[threadIdx.x + u * kOT] = c4[t0 + threadIdx.x + u * kOT];
     __syncthreads();
-    // Codes before ci count, equal ones only at a smaller index.
+    // Codes before a landmark's own count, equal ones only at a smaller index
+    // (i0 is even, so both landmarks lie in one group of four); codes have 30
+    // bits, so the sign of a difference tells.
 #pragma unroll 4
     for (int j = lane; j < len; j += kLanes) {
-      const uint4 c = tile[j];
-      const unsigned thr = ci + (4 * (t0 + j) + 3 < i ? 1u : 0u);
-      rank += (c.x < thr) + (c.y < thr) + (c.z < thr) + (c.w < thr);
+      const int4 c = tile[j];
+      const int lt = 4 * (t0 + j) + 3 < i0 ? 1 : 0;
+      const int h0 = c0 + lt, h1 = c1 + lt;
+      n0 += ((c.x - h0) >> 31) + ((c.y - h0) >> 31) + ((c.z - h0) >> 31) + ((c.w - h0) >> 31);
+      n1 += ((c.x - h1) >> 31) + ((c.y - h1) >> 31) + ((c.z - h1) >> 31) + ((c.w - h1) >> 31);
     }
   }
-  if (valid && (i >> 2) % kLanes == lane)
-    for (int j = i & ~3; j < i; ++j) rank += codes[j] == ci;
-#pragma unroll
-  for (int o = 1; o < kLanes; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-  if (i >= a.n && i < a.npad && lane < D) {  // the padding of the record slot
-    float* rec = reinterpret_cast<float*>(a.qp + (i >> 1) * D) + 2 * lane + (i & 1);
-    rec[0] = rec[2 * D] = 0.f;
+  n0 = -n0;
+  n1 = -n1;
+  if ((i0 >> 2) % kLanes == lane && i0 < a.n) {
+    for (int j = i0 & ~3; j < i0; ++j) n0 += static_cast<int>(codes[j]) == c0;
+    for (int j = i0 & ~3; j <= i0; ++j) n1 += static_cast<int>(codes[j]) == c1;
   }
-  if (!valid || lane >= D) return;
-  const int r = static_cast<int>(rank), k = lane;
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) {
+    n0 += __shfl_xor_sync(0xffffffffu, n0, o);
+    n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+  }
+  // Lanes 0..D-1 pack the first landmark's coordinates, lanes 4.. the second's.
+  const int i = i0 + lane / 4, k = lane % 4;
+  if (k >= D) return;
+  if (i >= a.n) {
+    if (i < a.npad) {  // the padding of the record slot
+      float* rec = reinterpret_cast<float*>(a.qp + (i >> 1) * D) + 2 * k + (i & 1);
+      rec[0] = rec[2 * D] = 0.f;
+    }
+    return;
+  }
+  const int r = lane / 4 ? n1 : n0;
   if (k == 0) perm[r] = i;
   const int src = D * i + k, dst = D * r + k;
   const float q = a.q[src];
@@ -197,7 +214,7 @@ cudaError_t launch_order_pack(const PackArgs& a, unsigned* codes, int* perm, uns
                               cudaStream_t st) {
   const size_t nbox4 = nbox / 4;
   const int grid = static_cast<int>(std::min<size_t>(std::max<size_t>((a.n + 31 + kOT) / kOT, nbox4 / (4 * kOT)), 1216));
-  const long long threads = static_cast<long long>(a.npad) * kLanes;
+  const long long threads = static_cast<long long>(a.npad) / 2 * kLanes;
   const int rgrid = static_cast<int>((threads + kOT - 1) / kOT);
   uint4* b4 = reinterpret_cast<uint4*>(boxes);
   const float kq = static_cast<float>(a.kq);

@@ -1,4 +1,4 @@
-"""Ordered sweeps (of 10^9 pairs and more: landmarks packed along a space-filling
+"""Ordered sweeps (of 8 evaluations and 10^9 pairs and more: landmarks packed along a space-filling
 curve, runs of sources whose Gaussian is exactly zero left out) against
 the same sweeps with every pair evaluated, which a launch-shape override selects.
 
@@ -57,14 +57,14 @@ def case(n, kind, dim):
 
 
 @pytest.mark.parametrize("n,kind,dim,T,kw", [
-    (16384, "surface", 3, 4, {}),
-    (12289, "islands", 3, 7, {"ckpt_every": 3}),
-    (18433, "points", 3, 3, {}),
+    (16384, "surface", 3, 8, {}),
+    (12289, "islands", 3, 8, {"ckpt_every": 3}),
+    (18433, "points", 3, 8, {}),
     (8255, "surface", 3, 4, {"integrator": "rk4", "h_at": "end"}),
-    (16001, "surface", 2, 4, {}),
+    (16001, "surface", 2, 8, {}),
     (16385, "islands", 2, 2, {"integrator": "rk4", "ckpt_every": 1}),
-    (16500, "surface", 3, 4, {"h_at": "end"}),
-    (70001, "islands", 3, 1, {}),
+    (16500, "surface", 3, 8, {"h_at": "end"}),
+    (70001, "islands", 3, 8, {}),
 ])
 def test_ordered_gradient_equals_every_pair(n, kind, dim, T, kw):
     q, p, t = case(n, kind, dim)
@@ -78,7 +78,7 @@ def test_ordered_gradient_equals_every_pair(n, kind, dim, T, kw):
 @pytest.mark.parametrize("n,dim", [(16511, 3), (16001, 2)])
 def test_ordered_flow_comes_back_in_the_callers_order(n, dim):
     q, p, _ = case(n, "surface", dim)
-    run = lambda: gs().shoot_forward(q, p, 4, 0.05)  # noqa: E731
+    run = lambda: gs().shoot_forward(q, p, 8, 0.05)  # noqa: E731
     a, b = run(), every_pair(run)
     bar = BAR + 2.0 ** -24 * float(q.abs().max()) * 0.85 / 0.05
     assert rel(a[0], b[0]) < bar and rel(a[1], b[1]) < bar and abs(a[2] - b[2]) < BAR * abs(b[2])
