@@ -483,8 +483,10 @@ int shoot_ckpt(const Workspace& w, const gs_params& prm) {
 // 233, 477, 493; planar (0.05, 0.1) N = 3000 28.2 against 23.8, 30.0; 4096 38.6
 // against 30.1, 38.1.  The order itself takes about 10 us a call: a sweep has 10^9
 // pairs (1 ms) at least, and 8 evaluations, as ranking the landmarks reads N^2
-// codes.  The rule must not depend on what a sweep computes:
-// register compares the positions of a flow with a gradient's targets.
+// codes.  A flow alone stays unordered (at sigma = 0.2 it took 1775 against 1714 us
+// at N = 16384, T = 10: the culling forward kernel has 64 registers for 55), except
+// where it must match a gradient (register compares its positions with the
+// gradient's targets) or many points follow it.
 bool use_order(int npad, int J, int dim) {
   return npad >= (dim == 2 ? kOrderNpad2 : kOrderNpad) && J >= 8 && static_cast<double>(J) * npad * npad >= 1e9 && (J + 1) * box_words(npad) * sizeof(unsigned) <= (size_t{1} << 30) && !step_override_set();
 }
@@ -569,7 +571,7 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
   pk.dim = dim;
   pk.npad = round_up(n, kPad);
   const int npad = pk.npad, J = stages_of(prm.integrator) * prm.T;
-  const bool ordered = use_order(npad, J, dim);
+  const bool ordered = (kind == 1 || out.order_flow) && use_order(npad, J, dim);
   if (ordered) {
     const size_t nbox = (J + 1) * box_words(npad);
     if ((s = reserve_order(w, npad, nbox)) != GS_OK) return s;

@@ -179,6 +179,7 @@ gs_status reserve_order(Workspace& w, int npad, size_t nbox);
 struct ShootOut {
   float *a = nullptr, *b = nullptr;  // kind 0: q(1), p(1); kind 1: dL/dp0, dL/dq0
   double* gp64 = nullptr;            // kind 1: FP64 dL/dp0
+  bool order_flow = false;           // kind 0: in spatial order where a gradient would be
 };
 // Enqueue one forward flow (kind 0) or gradient (kind 1) from inputs on the
 // device: momenta from p64_in (FP64) when set, else from dp.  Afterwards, in

@@ -580,7 +580,9 @@ gs_status run_register(const gs_params* prm, const float* q0, const float* targe
   bool dummy = false;
   if ((s = copy_out(p0_inout, w->out_a, n3, st, &dummy)) != GS_OK) return s;
   if (info) {
-    if ((s = enqueue_shoot(*w, 0, *prm, dq, nullptr, w->lb.x, nullptr, ShootOut{}, st)) != GS_OK) return s;
+    ShootOut flow;
+    flow.order_flow = true;  // q(1) in the order of the gradient's targets
+    if ((s = enqueue_shoot(*w, 0, *prm, dq, nullptr, w->lb.x, nullptr, flow, st)) != GS_OK) return s;
     GS_CUDA(vlaunch(grid, st, k_dist, (const double*)w->q64, (const double*)w->t64, n, dim_of(*prm), w->lb.part,
                     w->lb.ticket, w->lb.scal));
     double* const dist = w->lb.host;

@@ -412,13 +412,15 @@ extern "C" gs_status flow_points(const gs_params* prm, const float* q0, const fl
   // The forward flow: record slot k of the trajectory holds the landmark
   // state of step k.
   const KernelScales sc = make_scales(prm->sigma);
-  if ((s = enqueue_shoot(*w, 0, *prm, dq, dp, nullptr, nullptr, ShootOut{}, st)) != GS_OK) return s;
+  ShootOut flow;
+  flow.order_flow = m / 16 >= n;
+  if ((s = enqueue_shoot(*w, 0, *prm, dq, dp, nullptr, nullptr, flow, st)) != GS_OK) return s;
   // T Euler steps of the points, each with that step's landmark state.
   k_points_to64<<<conv_blocks(m3), 256, 0, st>>>(dx, w->pts64, m3);
   GS_CUDA(cudaGetLastError());
   const VelConfig c = vel_config(m, npad, w->num_sms);
   // The test of the runs takes about 1 us a CTA: worth it from 1024 landmarks a CTA.
-  const bool ordered = c.split_len >= 1024 && !small_path(*w, *prm) && use_order(npad, T, 3);
+  const bool ordered = flow.order_flow && c.split_len >= 1024 && !small_path(*w, *prm) && use_order(npad, T, 3);
   for (int k = 0; k < T; ++k) {
     VelArgs a{w->traj + static_cast<size_t>(k) * w->slot(), w->pts64, nullptr, nullptr, m, npad, c.split_len, sc.kq,
               1.0 / T, ordered ? w->boxes + k * box_words(npad) : nullptr, w->status};

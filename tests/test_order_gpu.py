@@ -76,7 +76,7 @@ def test_ordered_gradient_equals_every_pair(n, kind, dim, T, kw):
 
 
 @pytest.mark.parametrize("n,dim", [(16511, 3), (16001, 2)])
-def test_ordered_flow_comes_back_in_the_callers_order(n, dim):
+def test_flow_comes_back_in_the_callers_order(n, dim):
     q, p, _ = case(n, "surface", dim)
     run = lambda: gs().shoot_forward(q, p, 8, 0.05)  # noqa: E731
     a, b = run(), every_pair(run)
