@@ -571,7 +571,8 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
   pk.dim = dim;
   pk.npad = round_up(n, kPad);
   const int npad = pk.npad, J = stages_of(prm.integrator) * prm.T;
-  const bool ordered = (kind == 1 || out.order_flow) && use_order(npad, J, dim);
+  // (a flow in spatial order has no outputs: its state is read where it lies)
+  const bool ordered = (kind == 1 || (out.order_flow && !out.a && !out.b)) && use_order(npad, J, dim);
   if (ordered) {
     const size_t nbox = (J + 1) * box_words(npad);
     if ((s = reserve_order(w, npad, nbox)) != GS_OK) return s;
@@ -592,10 +593,7 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
       float* const o = f ? out.b : out.a;
       const double* const x = f ? w.p64 : w.q64;
       if (!o) continue;
-      if (ordered)
-        GS_CUDA(launch_unpack_perm(x, w.perm, o, n, dim, st));
-      else
-        GS_CUDA(launch_unpack(UnpackArgs{x, o, n3}, st));
+      GS_CUDA(launch_unpack(UnpackArgs{x, o, n3}, st));
     }
   } else {
     const size_t bytes = n3 * sizeof(float);

@@ -337,8 +337,6 @@ cudaError_t launch_unpack(const UnpackArgs& a, cudaStream_t st);
 // pairs are in reach; dense[0] is a ticket (zero between calls).
 cudaError_t launch_order_pack(const PackArgs& a, unsigned* codes, int* perm, unsigned* boxes, size_t nbox, int* dense,
                               cudaStream_t st);
-// out[perm[r]] = x64[r] as float32.
-cudaError_t launch_unpack_perm(const double* x64, const int* perm, float* out, int n, int dim, cudaStream_t st);
 // Restore an FP64 state checkpoint into q64, p64 and record slot 0 of rec,
 // with the same rounding as the step kernels' epilogue.
 cudaError_t launch_restore(const double* ckq, const double* ckp, double* q64, double* p64, float4* rec, int n,

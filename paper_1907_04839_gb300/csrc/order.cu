@@ -199,15 +199,6 @@ __global__ void __launch_bounds__(kOT) k_rank_pack(PackArgs a, const unsigned* c
   }
 }
 
-// out[perm[r]] = x64[r], row by row.
-template <int D>
-__global__ void __launch_bounds__(kOT) k_unpack_perm(const double* x64, const int* perm, float* out, int n) {
-  const int t = blockIdx.x * kOT + threadIdx.x;
-  if (t >= D * n) return;
-  const int r = t / D, k = t - D * r;
-  out[D * static_cast<size_t>(perm[r]) + k] = (float)x64[t];
-}
-
 }  // namespace
 
 cudaError_t launch_order_pack(const PackArgs& a, unsigned* codes, int* perm, unsigned* boxes, size_t nbox, int* dense,
@@ -236,15 +227,6 @@ cudaError_t launch_order_pack(const PackArgs& a, unsigned* codes, int* perm, uns
   const unsigned* const cc = codes;
   return a.dim == 2 ? cudaLaunchKernelEx(&cfg, k_rank_pack<2>, a, cc, perm, boxes, dense)
                     : cudaLaunchKernelEx(&cfg, k_rank_pack<3>, a, cc, perm, boxes, dense);
-}
-
-cudaError_t launch_unpack_perm(const double* x64, const int* perm, float* out, int n, int dim, cudaStream_t st) {
-  const int grid = (dim * n + kOT - 1) / kOT;
-  if (dim == 2)
-    k_unpack_perm<2><<<grid, kOT, 0, st>>>(x64, perm, out, n);
-  else
-    k_unpack_perm<3><<<grid, kOT, 0, st>>>(x64, perm, out, n);
-  return cudaGetLastError();
 }
 
 }  // namespace gs
