@@ -97,6 +97,8 @@ struct VelArgs {
   int m, npad, split_len;
   double kq, dt;
   const unsigned* box;  // boxes of the landmarks' runs (Cull)
+  const int* dense;     // set: nearly all pairs are in reach, and the steps of the flow that
+                        // made this state grew no boxes (null: the boxes stand)
   unsigned* status;
 };
 
@@ -172,7 +174,9 @@ __global__ void __launch_bounds__(kVT) k_velocity(VelArgs a) {
     const int nrun = a.npad / kGran;
     if (threadIdx.x < 32) {
       const int run = static_cast<int>(static_cast<long long>(threadIdx.x) * nrun / 32);
-      const bool all = __all_sync(0xffffffffu, in_reach(tb, run_box<3>(load_box(a.box, run))));
+      bool in = a.dense && *a.dense != 0;
+      if (!in) in = in_reach(tb, run_box<3>(load_box(a.box, run)));
+      const bool all = __all_sync(0xffffffffu, in);
       if (threadIdx.x == 0) list[kListCap] = all;
     }
     __syncthreads();
@@ -377,7 +381,8 @@ extern "C" gs_status velocity_field(int64_t N, int64_t M, double sigma, const fl
   w->clean_n = -1;  // record slot 0 was overwritten
   // The points are read and the velocities written where the caller keeps them.
   const VelConfig c = vel_config(m, npad, w->num_sms);
-  VelArgs a{w->traj, nullptr, dx, dv, m, npad, c.split_len, sc.kq, 0.0, ordered ? w->boxes : nullptr, w->status};
+  VelArgs a{w->traj, nullptr, dx, dv, m, npad, c.split_len, sc.kq, 0.0, ordered ? w->boxes : nullptr, nullptr,
+            w->status};
   GS_CUDA(launch_velocity(c, a, st, true));
   bool want_sync = host;
   if (dv != v && (s = copy_out(v, dv, m3, st, &want_sync)) != GS_OK) return s;
@@ -423,7 +428,8 @@ extern "C" gs_status flow_points(const gs_params* prm, const float* q0, const fl
   const bool ordered = flow.order_flow && c.split_len >= 1024 && !small_path(*w, *prm) && use_order(npad, T, 3);
   for (int k = 0; k < T; ++k) {
     VelArgs a{w->traj + static_cast<size_t>(k) * w->slot(), w->pts64, nullptr, nullptr, m, npad, c.split_len, sc.kq,
-              1.0 / T, ordered ? w->boxes + k * box_words(npad) : nullptr, w->status};
+              1.0 / T, ordered ? w->boxes + k * box_words(npad) : nullptr, ordered ? w->dense + 1 : nullptr,
+              w->status};
     GS_CUDA(launch_velocity(c, a, st, k > 0));
   }
   float* dx1 = nullptr;
