@@ -16,6 +16,7 @@
 // follows q(t).
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <mutex>
 #include <set>
 
@@ -356,6 +357,10 @@ extern "C" gs_status velocity_field(int64_t N, int64_t M, double sigma, const fl
   if ((s = stage_in(x, w->pts_in, m3, st, &dx, &host)) != GS_OK) return s;
   float* dv = nullptr;
   if ((s = out_ptr(v, w->pts_out, &dv)) != GS_OK) return s;
+  // A tile's velocities may be written before another tile's points are read:
+  // arrays that overlap other than point for point go through the buffer.
+  const auto at = [](const float* a) { return reinterpret_cast<uintptr_t>(a); };
+  if (dv != dx && at(dv) < at(dx + m3) && at(dx) < at(dv + m3)) dv = w->pts_out;
   const KernelScales sc = make_scales(sigma);
   // The order of the landmarks reads N codes per landmark and takes one launch
   // more: under 2 % of the pair sums from 64 points a landmark and 10^9 pairs
@@ -379,7 +384,8 @@ extern "C" gs_status velocity_field(int64_t N, int64_t M, double sigma, const fl
     GS_CUDA(launch_to_records(&qp, 1, n, npad, w->status, st));
   }
   w->clean_n = -1;  // record slot 0 was overwritten
-  // The points are read and the velocities written where the caller keeps them.
+  // The points are read and (apart from such overlaps) the velocities written
+  // where the caller keeps them.
   const VelConfig c = vel_config(m, npad, w->num_sms);
   VelArgs a{w->traj, nullptr, dx, dv, m, npad, c.split_len, sc.kq, 0.0, ordered ? w->boxes : nullptr, nullptr,
             w->status};
