@@ -666,7 +666,12 @@ gs_status run_step(int kind, int64_t N, double sigma, const float* q, const floa
   const int n = static_cast<int>(N), npad = round_up(n, kPad);
   const StepConfig c = choose_step_config(kind, npad, w->num_sms);
   if (c.threads == 0) return fail(GS_EINVAL, "no step kernel configuration");
-  if ((s = reserve(*w, npad, 1, 1)) != GS_OK) return s;
+  // The fused kernels' tiles are the grid's y: 65535 of 64 (or 128) landmarks.
+  // Past them the split-partial kernels, whose tiles are x, take any N.
+  const bool fused = c.tiles <= 65535;
+  PairConfig pc{};
+  if (!fused) pc = kind == 0 ? choose_forward_config(npad, w->num_sms) : choose_backward_config(npad, w->num_sms);
+  if ((s = reserve(*w, npad, 1, fused ? 1 : pc.splits)) != GS_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t n3 = 3 * static_cast<size_t>(n);
   bool host = false;
@@ -677,8 +682,8 @@ gs_status run_step(int kind, int64_t N, double sigma, const float* q, const floa
     if ((s = stage_in(alpha, w->in_a, n3, st, &da, &host)) != GS_OK) return s;
     if ((s = stage_in(beta, w->in_t, n3, st, &db, &host)) != GS_OK) return s;
   }
-  // Hp, Hq / dalpha, dbeta straight from a dry step of the fused kernels: the
-  // records, then the pair sums with their cluster reduction.
+  // The records, then the pair sums: Hp, Hq / dalpha, dbeta straight from a dry
+  // step of the fused kernels with their cluster reduction.
   float *o0 = nullptr, *o1 = nullptr;
   if ((s = out_ptr(out0, w->out_a, &o0)) != GS_OK) return s;
   if ((s = out_ptr(out1, w->out_b, &o1)) != GS_OK) return s;
@@ -686,7 +691,18 @@ gs_status run_step(int kind, int64_t N, double sigma, const float* q, const floa
   const RecordSet sets[2] = {{dq, dp, w->traj, sc.kq, 1.0, 0}, {da, db, w->adj, 1.0, sc.kappa, 1}};
   GS_CUDA(launch_to_records(sets, kind + 1, n, npad, w->status, st));
   w->clean_n = -1;  // traj slot 0 / adjoint arrays were overwritten
-  if (kind == 0) {
+  if (!fused) {
+    if (kind == 0) {
+      const PairFwdArgs a{w->traj, w->part, npad, pc.split_len, static_cast<float>(sc.kappa), w->status};
+      GS_CUDA(launch_pair_forward(pc, a, st, false));
+    } else {
+      const PairBwdArgs a{w->traj, w->adj, w->part, npad, pc.split_len, static_cast<float>(sc.kq),
+                          static_cast<float>(sc.kappa), w->status};
+      GS_CUDA(launch_pair_backward(pc, a, st, false));
+    }
+    // Partials hold (Hp, Hq) forward and (dalpha, dbeta) backward.
+    GS_CUDA(launch_partials_to_out(w->part, pc.splits, n, npad, kind == 0 ? o1 : o0, kind == 0 ? o0 : o1, st));
+  } else if (kind == 0) {
     StepFwdArgs a = forward_step_args(*w, c, 0, n, 1, 0, sigma, 0.0);
     a.dry = 1;
     a.out_q = o0;

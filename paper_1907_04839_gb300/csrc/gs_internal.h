@@ -84,6 +84,7 @@ struct PairConfig {
 };
 
 PairConfig choose_forward_config(int npad, int num_sms);
+PairConfig choose_backward_config(int npad, int num_sms);
 // A given kernel variant (threads per CTA, targets per thread); splits <= 0
 // picks the balanced split count.  threads == 0 in the result: no such variant.
 PairConfig forward_config_for(int npad, int num_sms, int threads, int R, int splits);

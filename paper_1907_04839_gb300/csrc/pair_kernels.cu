@@ -211,6 +211,7 @@ PairConfig balanced_config(int npad, int num_sms, int threads, int R, int occ) {
 }
 
 constexpr int kFwdNT = 64, kFwdR = 4;
+constexpr int kBwdNT = 64, kBwdR = 2;
 
 }  // namespace
 
@@ -244,6 +245,10 @@ PairConfig choose_forward_config_capped(int npad, int num_sms, int max_splits) {
   PairConfig c = choose_forward_config(npad, num_sms);
   if (c.splits > max_splits) set_splits(c, npad, max_splits);
   return c;
+}
+
+PairConfig choose_backward_config(int npad, int num_sms) {
+  return backward_config_for(npad, num_sms, kBwdNT, kBwdR, 0);
 }
 
 cudaError_t launch_pair_forward(const PairConfig& cfg, const PairFwdArgs& a, cudaStream_t st, bool pdl) {
