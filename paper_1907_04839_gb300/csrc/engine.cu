@@ -457,6 +457,16 @@ gs_status get_graph(Workspace& w, const GraphKey& key, cudaGraphExec_t* out) {
   return GS_OK;
 }
 
+// Whether the stream is being captured into a graph (no allocation then).
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return c != cudaStreamCaptureStatusNone;
+}
+
 // Small problems go through one launch per call (small.cu).  The line: a forward
 // and a reverse step take 1.8 us at N = 64, 3.9 at 256, 7.5 at 512 in one launch
 // and 9.3 us by launches per step at 576 (8.4 at 256), whose gradient ends up
@@ -472,8 +482,39 @@ bool small_path(const Workspace& w, const gs_params& prm) {
   return use_small(w, round_up(prm.N, kPad), stages_of(prm.integrator) * prm.T);
 }
 
-int shoot_ckpt(const Workspace& w, const gs_params& prm) {
-  return small_path(w, prm) ? 0 : effective_ckpt(prm.ckpt_every, prm.T);
+// float4 of the trajectory that a one-launch gradient of prm keeps.
+static size_t small_traj_f4(const gs_params& prm) {
+  const size_t slot = static_cast<size_t>(round_up(prm.N, kPad)) / 2 * dim_of(prm);
+  return (static_cast<size_t>(stages_of(prm.integrator)) * prm.T + 1) * slot;
+}
+
+// Room for it; false where there is none, or where the caller's stream is
+// being captured.
+static bool reserve_small(Workspace& w, size_t f4, cudaStream_t st) {
+  if (f4 <= w.cap_small) return true;
+  if (capturing(st)) return false;
+  cudaFree(w.small_traj);
+  w.small_traj = nullptr;
+  w.cap_small = 0;
+  void* v = nullptr;
+  if (cudaMalloc(&v, f4 * sizeof(float4) + 256) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  w.small_traj = static_cast<float4*>(v);
+  w.cap_small = f4;
+  return true;
+}
+
+gs_status reserve_sweep(Workspace& w, int kind, const gs_params& prm, int slots, cudaStream_t st) {
+  const int npad = round_up(prm.N, kPad), ckpt = kind == 1 ? effective_ckpt(prm.ckpt_every, prm.T) : 0;
+  if (ckpt && small_path(w, prm)) {
+    const gs_status s = reserve(w, npad, std::max(slots, 1), 1, 0);
+    if (s != GS_OK) return s;
+    if (reserve_small(w, small_traj_f4(prm), st)) return GS_OK;
+  }
+  return reserve(w, npad, std::max(slots, record_slots(prm.T, ckpt, stages_of(prm.integrator))), 1,
+                 ckpt ? (prm.T + ckpt - 1) / ckpt : 0);
 }
 
 // Larger problems are packed in spatial order, so that the step kernels can
@@ -525,7 +566,10 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
   gs_status s = ensure_clean(w, n, st, dim);
   if (s != GS_OK) return s;
   const KernelScales sc = make_scales(prm.sigma);
-  if (small_path(w, prm)) {
+  const int npad = round_up(n, kPad), J = stages_of(prm.integrator) * prm.T;
+  // (see reserve_sweep; without the room the gradient runs by launches per step)
+  const bool own_traj = kind == 1 && effective_ckpt(prm.ckpt_every, prm.T) > 0;
+  if (small_path(w, prm) && (!own_traj || small_traj_f4(prm) <= w.cap_small)) {
     SmallArgs a;
     a.q = dq;
     a.p = dp;
@@ -533,7 +577,7 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
     a.tgt = kind == 1 ? dt : nullptr;
     a.kind = kind;
     a.n = n;
-    a.npad = round_up(n, kPad);
+    a.npad = npad;
     a.T = prm.T;
     a.groups = 0;
     a.rk = prm.integrator == GS_RK4;
@@ -543,8 +587,8 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
     a.kappa = sc.kappa;
     a.lambda = prm.lambda;
     a.adj_scale = a.rk ? a.dt / 6.0 : 1.0;
-    a.traj = w.traj;
-    a.slot = w.slot();
+    a.traj = own_traj ? w.small_traj : w.traj;
+    a.slot = own_traj ? static_cast<size_t>(npad) / 2 * dim : w.slot();
     a.q64 = w.q64;
     a.p64 = w.p64;
     a.t64 = kind == 1 ? w.t64 : nullptr;
@@ -569,8 +613,7 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
   pk.kq = sc.kq;
   pk.status = w.status;
   pk.dim = dim;
-  pk.npad = round_up(n, kPad);
-  const int npad = pk.npad, J = stages_of(prm.integrator) * prm.T;
+  pk.npad = npad;
   // (a flow in spatial order has no outputs: its state is read where it lies)
   const bool ordered = (kind == 1 || (out.order_flow && !out.a && !out.b)) && use_order(npad, J, dim);
   if (ordered) {
@@ -623,13 +666,9 @@ gs_status run_shoot(int kind, const gs_params* prm, const float* q0, const float
   std::lock_guard<std::mutex> lk(g_mu);
   Workspace* w = nullptr;
   if ((s = get_workspace(&w)) != GS_OK) return s;
-  const int n = static_cast<int>(prm->N), T = prm->T;
-  const int npad = round_up(n, kPad);
-  const int ckpt = kind == 1 ? shoot_ckpt(*w, *prm) : 0;
-  if ((s = reserve(*w, npad, record_slots(T, ckpt, stages_of(prm->integrator)), 1, ckpt ? (T + ckpt - 1) / ckpt : 0)) !=
-      GS_OK)
-    return s;
+  const int n = static_cast<int>(prm->N);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if ((s = reserve_sweep(*w, kind, *prm, 0, st)) != GS_OK) return s;
   const int dim = dim_of(*prm);
   const size_t n3 = static_cast<size_t>(dim) * n;  // floats per (N, dim) array
   bool host = false;

@@ -117,6 +117,12 @@ struct Workspace {
   std::vector<void*> ord_allocs;
   int *perm = nullptr, *dense = nullptr;
   unsigned *codes = nullptr, *boxes = nullptr;
+  // Trajectory of a one-launch gradient (small.cu) whose caller asked for
+  // checkpoints, in slots of the problem's own size: 50 MB at most (kSmallSteps,
+  // kSmallNpad), where slots of traj are as large as the largest problem's.
+  // Grown on demand.
+  size_t cap_small = 0;
+  float4* small_traj = nullptr;
   // Query points of velocity_field / flow_points (grown on demand).
   int cap_pts = 0;
   std::vector<void*> pt_allocs;
@@ -139,6 +145,9 @@ struct Workspace {
     ord_allocs.clear();
     cap_ord = 0;
     cap_box = 0;
+    cudaFree(small_traj);
+    small_traj = nullptr;
+    cap_small = 0;
     cap_npad = cap_T = cap_splits = cap_red = cap_ck = 0;
     clean_n = -1;
   }
@@ -150,6 +159,9 @@ gs_status get_workspace(Workspace** out);
 // Room for npad landmarks, record slots 0..T, the split partials and nck
 // FP64 state checkpoints.
 gs_status reserve(Workspace& w, int npad, int T, int splits, int nck = 0);
+// Room for a flow (kind 0) or gradient (kind 1) of prm, and for `slots` record
+// slots at least.
+gs_status reserve_sweep(Workspace& w, int kind, const gs_params& prm, int slots, cudaStream_t st);
 gs_status ensure_clean(Workspace& w, int n, cudaStream_t st, int dim = 3);
 // True for memory the current device can use in place: its own device
 // memory or managed memory.
@@ -164,11 +176,9 @@ gs_status out_ptr(float* user, float* staging, float** dev);
 gs_status finish_sync(Workspace& w, cudaStream_t st);
 gs_status check_params(const gs_params* prm);
 gs_status get_graph(Workspace& w, const GraphKey& key, cudaGraphExec_t* out);
-// Whether a flow or gradient of prm runs as one launch (small.cu), and the
-// checkpoint interval of its reverse sweep (0 on the small path, whose
-// trajectory is at most a few MB).
+// Whether a flow or gradient of prm runs as one launch (small.cu), which keeps
+// the whole trajectory whatever the checkpoint interval.
 bool small_path(const Workspace& w, const gs_params& prm);
-int shoot_ckpt(const Workspace& w, const gs_params& prm);
 // Whether a sweep of J evaluations packs its landmarks in spatial order
 // (order.cu); the words of the boxes of one state; room for the order
 // of npad landmarks and nbox words of boxes.

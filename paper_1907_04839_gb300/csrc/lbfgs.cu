@@ -557,15 +557,11 @@ gs_status run_register(const gs_params* prm, const float* q0, const float* targe
   std::lock_guard<std::mutex> lk(engine_mutex());
   Workspace* w = nullptr;
   if ((s = get_workspace(&w)) != GS_OK) return s;
-  const int n = static_cast<int>(prm->N), npad = round_up(n, kPad), n3 = dim_of(*prm) * n;
-  const int ckpt = shoot_ckpt(*w, *prm);
-  const int S = stages_of(prm->integrator);
-  if ((s = reserve(*w, npad, std::max(S * prm->T, record_slots(prm->T, ckpt, S)), 1,
-                   ckpt ? (prm->T + ckpt - 1) / ckpt : 0)) !=
-      GS_OK)
-    return s;
-  if ((s = alloc_lbfgs(*w, n3, prm->lbfgs_m)) != GS_OK) return s;
+  const int n = static_cast<int>(prm->N), n3 = dim_of(*prm) * n;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // (the flow at the end keeps every state)
+  if ((s = reserve_sweep(*w, 1, *prm, stages_of(prm->integrator) * prm->T, st)) != GS_OK) return s;
+  if ((s = alloc_lbfgs(*w, n3, prm->lbfgs_m)) != GS_OK) return s;
   bool host = false;
   const float *dq = nullptr, *dt = nullptr, *dp = nullptr;
   if ((s = stage_in(q0, w->in_q, n3, st, &dq, &host)) != GS_OK) return s;
