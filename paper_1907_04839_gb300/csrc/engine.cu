@@ -532,32 +532,30 @@ bool use_order(int npad, int J, int dim) {
   return npad >= (dim == 2 ? kOrderNpad2 : kOrderNpad) && J >= 8 && static_cast<double>(J) * npad * npad >= 1e9 && (J + 1) * box_words(npad) * sizeof(unsigned) <= (size_t{1} << 30) && !step_override_set();
 }
 
-gs_status reserve_order(Workspace& w, int npad, size_t nbox) {
-  if (npad <= w.cap_ord && nbox <= w.cap_box) return GS_OK;
+bool reserve_order(Workspace& w, int npad, size_t nbox, cudaStream_t st) {
+  if (npad <= w.cap_ord && nbox <= w.cap_box) return true;
+  if (capturing(st)) return false;
   const int cn = std::max(npad, w.cap_ord);
   const size_t cb = std::max(nbox, w.cap_box);
-  w.drop_graphs();
-  for (void* p : w.ord_allocs) cudaFree(p);
-  w.ord_allocs.clear();
-  w.cap_ord = 0;
-  w.cap_box = 0;
+  if (w.cap_ord) w.drop_graphs();  // they hold the old buffers
+  w.free_order();
   const auto get = [&](auto** p, size_t count) {
     void* v = nullptr;
-    const cudaError_t e = cudaMalloc(&v, count * sizeof(**p) + 256);
-    if (e != cudaSuccess) return e;
+    if (cudaMalloc(&v, count * sizeof(**p) + 256) != cudaSuccess) return false;
     w.ord_allocs.push_back(v);
     *p = static_cast<std::remove_reference_t<decltype(*p)>>(v);
-    return e;
+    return true;
   };
-  GS_CUDA(get(&w.perm, cn));
-  GS_CUDA(get(&w.codes, cn));
-  GS_CUDA(get(&w.boxes, cb));
-  GS_CUDA(get(&w.dense, 2));
-  GS_CUDA(cudaMemset(w.dense, 0, 2 * sizeof(int)));
-  GS_CUDA(cudaDeviceSynchronize());  // the caller's stream need not wait for the default one
+  if (!get(&w.perm, cn) || !get(&w.codes, cn) || !get(&w.boxes, cb) || !get(&w.dense, 2) ||
+      cudaMemset(w.dense, 0, 2 * sizeof(int)) != cudaSuccess ||
+      cudaDeviceSynchronize() != cudaSuccess) {  // the caller's stream need not wait for the default one
+    cudaGetLastError();
+    w.free_order();
+    return false;
+  }
   w.cap_ord = cn;
   w.cap_box = cb;
-  return GS_OK;
+  return true;
 }
 
 gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const float* dq, const float* dp,
@@ -569,6 +567,7 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
   const int npad = round_up(n, kPad), J = stages_of(prm.integrator) * prm.T;
   // (see reserve_sweep; without the room the gradient runs by launches per step)
   const bool own_traj = kind == 1 && effective_ckpt(prm.ckpt_every, prm.T) > 0;
+  w.ordered = false;
   if (small_path(w, prm) && (!own_traj || small_traj_f4(prm) <= w.cap_small)) {
     SmallArgs a;
     a.q = dq;
@@ -615,10 +614,11 @@ gs_status enqueue_shoot(Workspace& w, int kind, const gs_params& prm, const floa
   pk.dim = dim;
   pk.npad = npad;
   // (a flow in spatial order has no outputs: its state is read where it lies)
-  const bool ordered = (kind == 1 || (out.order_flow && !out.a && !out.b)) && use_order(npad, J, dim);
+  const size_t nbox = (J + 1) * box_words(npad);
+  const bool ordered = (kind == 1 || (out.order_flow && !out.a && !out.b)) && use_order(npad, J, dim) &&
+                       reserve_order(w, npad, nbox, st);
+  w.ordered = ordered;
   if (ordered) {
-    const size_t nbox = (J + 1) * box_words(npad);
-    if ((s = reserve_order(w, npad, nbox)) != GS_OK) return s;
     GS_CUDA(launch_order_pack(pk, w.codes, w.perm, w.boxes, nbox, w.dense, st));
   } else {
     GS_CUDA(launch_pack(pk, st));
@@ -805,7 +805,7 @@ gs_status time_pair_kernels(const gs_params* prm, const float* q0, const float* 
   if (launches)
     *launches = small_path(*w, *prm) ? 1
                                      : 2 * stages_of(prm->integrator) * T + 1 + (prm->kinetic_at == GS_KINETIC_END ? 1 : 0) +
-                                           (use_order(npad, stages_of(prm->integrator) * T, 3) ? 1 : 0);
+                                           (w->ordered ? 1 : 0);
   return finish_sync(*w, st);
 }
 

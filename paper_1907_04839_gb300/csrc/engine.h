@@ -117,6 +117,7 @@ struct Workspace {
   std::vector<void*> ord_allocs;
   int *perm = nullptr, *dense = nullptr;
   unsigned *codes = nullptr, *boxes = nullptr;
+  bool ordered = false;  // whether the last sweep enqueued lies in spatial order
   // Trajectory of a one-launch gradient (small.cu) whose caller asked for
   // checkpoints, in slots of the problem's own size: 50 MB at most (kSmallSteps,
   // kSmallNpad), where slots of traj are as large as the largest problem's.
@@ -133,6 +134,12 @@ struct Workspace {
     for (auto& kv : graphs) cudaGraphExecDestroy(kv.second);
     graphs.clear();
   }
+  void free_order() {
+    for (void* p : ord_allocs) cudaFree(p);
+    ord_allocs.clear();
+    cap_ord = 0;
+    cap_box = 0;
+  }
   void free_all() {
     drop_graphs();
     for (void* p : allocs) cudaFree(p);
@@ -141,10 +148,7 @@ struct Workspace {
     for (void* p : pt_allocs) cudaFree(p);
     pt_allocs.clear();
     cap_pts = 0;
-    for (void* p : ord_allocs) cudaFree(p);
-    ord_allocs.clear();
-    cap_ord = 0;
-    cap_box = 0;
+    free_order();
     cudaFree(small_traj);
     small_traj = nullptr;
     cap_small = 0;
@@ -181,10 +185,12 @@ gs_status get_graph(Workspace& w, const GraphKey& key, cudaGraphExec_t* out);
 bool small_path(const Workspace& w, const gs_params& prm);
 // Whether a sweep of J evaluations packs its landmarks in spatial order
 // (order.cu); the words of the boxes of one state; room for the order
-// of npad landmarks and nbox words of boxes.
+// of npad landmarks and nbox words of boxes (false: there is none, or the
+// caller's stream is being captured and nothing can be allocated; the call then
+// keeps the caller's order).
 bool use_order(int npad, int J, int dim);
 size_t box_words(int npad);
-gs_status reserve_order(Workspace& w, int npad, size_t nbox);
+bool reserve_order(Workspace& w, int npad, size_t nbox, cudaStream_t st);
 // Device destinations of a sweep's results; null: not wanted.
 struct ShootOut {
   float *a = nullptr, *b = nullptr;  // kind 0: q(1), p(1); kind 1: dL/dp0, dL/dq0

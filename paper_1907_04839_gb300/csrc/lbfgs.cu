@@ -577,7 +577,7 @@ gs_status run_register(const gs_params* prm, const float* q0, const float* targe
   if ((s = copy_out(p0_inout, w->out_a, n3, st, &dummy)) != GS_OK) return s;
   if (info) {
     ShootOut flow;
-    flow.order_flow = true;  // q(1) in the order of the gradient's targets
+    flow.order_flow = w->ordered;  // q(1) in the order of the last gradient's targets
     if ((s = enqueue_shoot(*w, 0, *prm, dq, nullptr, w->lb.x, nullptr, flow, st)) != GS_OK) return s;
     GS_CUDA(vlaunch(grid, st, k_dist, (const double*)w->q64, (const double*)w->t64, n, dim_of(*prm), w->lb.part,
                     w->lb.ticket, w->lb.scal));

@@ -365,9 +365,9 @@ extern "C" gs_status velocity_field(int64_t N, int64_t M, double sigma, const fl
   // The order of the landmarks reads N codes per landmark and takes one launch
   // more: under 2 % of the pair sums from 64 points a landmark and 10^9 pairs
   // (350 us) on.
-  const bool ordered = npad >= 1024 && m / 64 >= n && static_cast<double>(n) * m >= 1e9;
+  const bool ordered = npad >= 1024 && m / 64 >= n && static_cast<double>(n) * m >= 1e9 &&
+                       reserve_order(*w, npad, box_words(npad), st);
   if (ordered) {
-    if ((s = reserve_order(*w, npad, box_words(npad))) != GS_OK) return s;
     PackArgs pk{};
     pk.q = dq;
     pk.p = dp;
@@ -431,7 +431,7 @@ extern "C" gs_status flow_points(const gs_params* prm, const float* q0, const fl
   GS_CUDA(cudaGetLastError());
   const VelConfig c = vel_config(m, npad, w->num_sms);
   // The test of the runs takes about 1 us a CTA: worth it from 1024 landmarks a CTA.
-  const bool ordered = flow.order_flow && c.split_len >= 1024 && !small_path(*w, *prm) && use_order(npad, T, 3);
+  const bool ordered = w->ordered && c.split_len >= 1024;
   for (int k = 0; k < T; ++k) {
     VelArgs a{w->traj + static_cast<size_t>(k) * w->slot(), w->pts64, nullptr, nullptr, m, npad, c.split_len, sc.kq,
               1.0 / T, ordered ? w->boxes + k * box_words(npad) : nullptr, ordered ? w->dense + 1 : nullptr,
