@@ -28,6 +28,11 @@ enum : unsigned {
   kErrBadLaunch = 4u,  // a kernel saw an inconsistent launch configuration
 };
 
+// Whether an evaluation that is thrown away may take its status word with it: a
+// non-finite value goes with the point it came from; an expired wait or a bad
+// launch is an error of the call.
+inline bool goes_with_its_point(unsigned status) { return (status & ~kErrNonFinite) == 0; }
+
 constexpr int kPad = 64;      // landmark padding granule
 constexpr int kChunk = 128;   // sources staged in shared memory per bulk copy
 constexpr int kStages = 4;    // chunk buffers in flight per CTA

@@ -497,8 +497,8 @@ struct Lbfgs {
       da.accept = kAcceptNone;
       double dphi0 = b.host[kRbSlope0];
       if (!(dphi0 < 0.0)) {  // not a descent direction: restart from -g
-        if (static_cast<unsigned>(b.host[kRbStatus]) & kErrNonFinite)
-          GS_CUDA(cudaMemsetAsync(w.status, 0, sizeof(unsigned), st));  // of the point thrown away
+        if (!goes_with_its_point(static_cast<unsigned>(b.host[kRbStatus]))) return finish_sync(w, st);
+        if (b.host[kRbStatus] != 0.0) GS_CUDA(cudaMemsetAsync(w.status, 0, sizeof(unsigned), st));
         dphi0 = -gnorm * gnorm;
         da.stored = stored = 0;
         if ((s = launch_direction(da)) != GS_OK) return s;
