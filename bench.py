@@ -620,7 +620,7 @@ def measure_velocity(gsh, reps=5, T=T_STEPS, peak=None):
         "flow_points_ms": t_flow, "point_steps_per_s": m * T / (t_flow * 1e-3),
         "flow_pair_interactions_per_s": T * pairs_vel / (t_flow * 1e-3),
         "velocity_field_ms": t_vel, "velocity_pair_interactions_per_s": pairs_vel / (t_vel * 1e-3),
-        "roofline": {"bound": "alu", "kernel": "k_velocity (one velocity_field call, conversions included)",
+        "roofline": {"bound": "alu", "kernel": "k_velocity (one velocity_field call; every pair counted, those out of reach left out)",
                      "achieved": tf, "peak": peak, "unit": "TFLOP/s", "frac": tf / peak,
                      "fp32_pipe_frac": INSTR_PER_PAIR_VEL * pairs_vel / (t_vel * 1e-3) / (peak * 1e12 / 2)},
         "timing": "CUDA events on the stream, device inputs, median of %d calls" % reps,

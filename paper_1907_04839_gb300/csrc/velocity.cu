@@ -244,7 +244,7 @@ __global__ void k_points_to32(const double* x64, float* x, size_t n3) {
 
 int conv_blocks(size_t n3) { return static_cast<int>(std::min<size_t>((n3 + 255) / 256, 4096)); }
 
-// Launch shape: tiles of 128 points; the cluster size C (a power of two,
+// Launch shape: tiles of kVM = 256 points; the cluster size C (a power of two,
 // at most 16) splits the landmarks so that the grid reaches about two
 // waves when the points alone do not.
 struct VelConfig {
